@@ -63,8 +63,7 @@ struct SharedHead {
     uint32_t rem_draws[2][kMaxRemnants]; // its draw counter
     double rem_t[2][kMaxRemnants];       // its time
     double inv_sigma[PF_MAX_OBS_DIM];  // 1 / sigma_p, correctly rounded
-    ZigX zig;                 // ziggurat layer edges
-    const ZigTab *zig_g;      // the full ziggurat table (global memory)
+    const ZigTab *zig_g;      // the ziggurat table (global memory)
     // exchange slot of a filter split over a thread-block cluster: each
     // block's share, read by the others through distributed shared memory
     double cx_lmax, cx_lsum;
@@ -150,19 +149,29 @@ __device__ __forceinline__ double propensity_reg(double rate, int desc, const La
 // as signed integers, so these compares run on the integer pipes.
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 
-// Simulate every particle of the filter from t_prev to t_end by Gillespie's
-// direct method (Supp. I, "Simulate X_t"; Sec. "The stochastic birth-death
+}  // namespace dev
+}  // namespace pf
+#include "ssa_fast.cuh"
+namespace pf {
+namespace dev {
+
+// Simulate N particles of the filter -- slots 0..N-1, or those `list` names --
+// from t_prev to t_end by Gillespie's direct method (Supp. I, "Simulate X_t"; Sec. "The stochastic birth-death
 // Model": SSA).  Lanes take particle slots from a pool in index order; each
 // loop trip is one direct-method step of every active lane.  Failure is
 // reported through sh.status (PF_ST_BUDGET when a particle needed more than
 // `budget` draws); `fired` counts reactions.  Particle slot j of `xs` is
 // particle j0 + j of the filter (j0 > 0 when the filter is split over the
 // blocks of a cluster); the random stream is keyed by the latter.
+//
+// This is the definition of the simulated law's outcome.  ssa_fast takes the
+// same decisions without FP64 and leaves here the particles it cannot decide,
+// and the intervals outside its conditions.
 template <int RM, int UM>
-__device__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N,
+__device__ __noinline__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N, const int *list,
                              double t_prev, double t_end, uint32_t key0, uint32_t key1,
                              uint32_t lane, uint32_t mrow, uint64_t budget,
-                             unsigned long long &fired, uint32_t j0 = 0) {
+                             unsigned long long &fired, uint32_t j0) {
     const int R = sh.net.R, U = sh.net.U;
     const uint32_t all = (R >= 32) ? 0xFFFFFFFFu : ((1u << R) - 1u);
     const long long t_end_bits = dbits(t_end);
@@ -185,7 +194,7 @@ __device__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N,
     auto take = [&](bool &act) {
         const int slot = atomicAdd(&sh.pool_next, 1);
         act = slot < N;
-        L.j = act ? slot : 0;
+        L.j = act ? (list ? list[slot] : slot) : 0;
         load_x(act);
     };
     double a[RM], S[RM];
@@ -318,7 +327,7 @@ __device__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N,
             const uint64_t r0 = (static_cast<uint64_t>(w.w1) << 32) | w.w0;
             const uint64_t r1 = (static_cast<uint64_t>(w.w3) << 32) | w.w2;
             double E;
-            const bool fast = zig_fast(r0, sh.zig.x, E);
+            const bool fast = zig_fast(r0, sh.zig_g->x, E);
             double run;
             if constexpr (kDepList) {
                 // The prefix sums below the earliest recomputed propensity of
@@ -359,7 +368,7 @@ __device__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N,
                 // path: the whole algorithm again from the first word)
                 if (!fast)
                     E = zig_exp(r0, draws, j0 + static_cast<uint32_t>(L.j), lane, mrow, key0, key1,
-                                sh.zig.x, sh.zig_g);
+                                sh.zig_g->x, sh.zig_g);
                 ++draws;
                 const double tau = div_pos(E, a0);
                 const double t_next = __dadd_rn(t, tau);
@@ -427,6 +436,38 @@ __device__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N,
         __syncthreads();
         src = dst;
         first = false;
+    }
+}
+
+// One interval's simulation by the whole block; `redo` is scratch for N slots.
+template <int RM, int UM>
+__device__ __forceinline__ void simulate(SharedHead &sh, bool fast, FastShared &fs, int *cols, int *xs,
+                                         int Np, int N, int *redo, double t_prev, double t_end,
+                                         uint32_t key0, uint32_t key1, uint32_t lane, uint32_t mrow,
+                                         uint64_t budget, unsigned long long &fired, uint32_t j0) {
+    const int tid = threadIdx.x;
+    if (fast) fast = fast_interval(fs, sh.net, sh.rate, xs, Np, N, t_prev, t_end, budget);
+    if (tid == 0) {
+        sh.pool_next = fast ? static_cast<int>(blockDim.x) : 0;
+        sh.rem_n[0] = 0;
+        sh.rem_n[1] = 0;
+    }
+    __syncthreads();
+    if (!fast) {
+        ssa_interval<RM, UM>(sh, xs, Np, N, nullptr, t_prev, t_end, key0, key1, lane, mrow, budget, fired, j0);
+        return;
+    }
+    ssa_fast<RM>(sh, fs, cols, xs, Np, N, key0, key1, lane, mrow, budget, fired, j0, redo);
+    __syncthreads();
+    const int again = fs.n_exact;
+    if (again > 0) {
+        if (tid == 0) {
+            sh.pool_next = 0;
+            sh.rem_n[0] = 0;
+            sh.rem_n[1] = 0;
+        }
+        __syncthreads();
+        ssa_interval<RM, UM>(sh, xs, Np, again, redo, t_prev, t_end, key0, key1, lane, mrow, budget, fired, j0);
     }
 }
 
@@ -694,10 +735,12 @@ struct FilterJob {
 };
 
 template <int RM, int UM>
-__device__ void run_filter(const FilterJob &job, SharedHead &sh, unsigned char *arrays) {
+__device__ void run_filter(const FilterJob &job, SharedHead &sh, bool fast, FastShared &fs, int *cols,
+                           unsigned char *arrays) {
     const int tid = threadIdx.x, B = blockDim.x;
     const int U = sh.net.U, P = sh.net.P;
     const int N = job.N, K = job.K;
+    if (fast) fast_network(fs, cols, sh.net);
     filter_setup(job.theta, sh);
     if (!sh.valid) {
         if (tid == 0) {
@@ -800,14 +843,8 @@ __device__ void run_filter(const FilterJob &job, SharedHead &sh, unsigned char *
             // the pool hands out particle slots in index order (the refill
             // loop and the tail consolidation absorb their unequal costs;
             // sorting them heaviest first no longer paid for its two passes)
-            if (tid == 0) {
-                sh.pool_next = 0;
-                sh.rem_n[0] = 0;
-                sh.rem_n[1] = 0;
-            }
-            __syncthreads();
-            ssa_interval<RM, UM>(sh, xs, Np, N, t_prev, t_k, key0, key1, lane, m32, job.budget,
-                                 fired);
+            simulate<RM, UM>(sh, fast, fs, cols, xs, Np, N, order, t_prev, t_k, key0, key1, lane, m32,
+                             job.budget, fired, 0u);
         }
         __syncthreads();
         if (want_ph) {
@@ -903,7 +940,8 @@ __host__ __device__ __forceinline__ size_t cluster_share_bytes(int N, int C, int
 // values after a cluster barrier, so all blocks pass the same barriers.
 // Requires n >= 1 in every block (N > (C - 1) ceil(N / C)); checked by the host.
 template <int RM, int UM>
-__device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, unsigned char *arrays) {
+__device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fast, FastShared &fs,
+                                   int *cols, unsigned char *arrays) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int C = static_cast<int>(cl.num_blocks());
@@ -914,6 +952,7 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, unsigne
     const int Np = (N + C - 1) / C;
     const int j0 = rank * Np;
     const int n = min(Np, N - j0);
+    if (fast) fast_network(fs, cols, sh.net);
     filter_setup(job.theta, sh);
     if (!sh.valid) {           // the same row in every block: all leave here
         if (tid == 0 && rank == 0) {
@@ -991,14 +1030,8 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, unsigne
 
         const double t_k = job.obs_times[k];
         if (t_k > t_prev) {
-            if (tid == 0) {
-                sh.pool_next = 0;
-                sh.rem_n[0] = 0;
-                sh.rem_n[1] = 0;
-            }
-            __syncthreads();
-            ssa_interval<RM, UM>(sh, xs, Np, n, t_prev, t_k, key0, key1, lane, m32, job.budget,
-                                 fired, static_cast<uint32_t>(j0));
+            simulate<RM, UM>(sh, fast, fs, cols, xs, Np, n, order, t_prev, t_k, key0, key1, lane, m32,
+                             job.budget, fired, static_cast<uint32_t>(j0));
         }
         __syncthreads();
 

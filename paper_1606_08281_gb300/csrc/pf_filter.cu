@@ -55,7 +55,9 @@ __global__ void __launch_bounds__(128, 4) filter_kernel(const FilterArgs args) {
         uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
         for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
     }
-    load_zig_table(sh.zig, args.zig);
+    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
+    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
+    if (args.fast) load_fast_zig(fs, args.zig);
     if (tid == 0) sh.zig_g = args.zig;
     __syncthreads();
     FilterJob job;
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(128, 4) filter_kernel(const FilterArgs args) {
     job.acc = args.acc ? args.acc + mrow : nullptr;
     job.reject_below = args.reject_below;
     job.slack = args.slack;
-    run_filter<RM, UM>(job, sh, smem);
+    run_filter<RM, UM>(job, sh, args.fast != 0, fs, cols, smem + args.fast);
 }
 
 // A filter split over the C blocks of a thread-block cluster (cluster size
@@ -99,7 +101,9 @@ __global__ void __launch_bounds__(128, 4) filter_kernel_cluster(const FilterArgs
         uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
         for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
     }
-    load_zig_table(sh.zig, args.zig);
+    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
+    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
+    if (args.fast) load_fast_zig(fs, args.zig);
     if (tid == 0) sh.zig_g = args.zig;
     __syncthreads();
     FilterJob job;
@@ -122,7 +126,7 @@ __global__ void __launch_bounds__(128, 4) filter_kernel_cluster(const FilterArgs
     job.acc = args.acc ? args.acc + mrow : nullptr;
     job.reject_below = args.reject_below;
     job.slack = args.slack;
-    run_filter_cluster<RM, UM>(job, sh, smem);
+    run_filter_cluster<RM, UM>(job, sh, args.fast != 0, fs, cols, smem + args.fast);
 }
 
 // Populations too large for shared memory: a grid of resident blocks walks
@@ -132,6 +136,7 @@ template <int RM, int UM>
 __global__ void __launch_bounds__(128, 4) filter_kernel_global(const FilterArgs args,
                                                                unsigned char *slabs,
                                                                size_t slab_bytes) {
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SharedHead sh;
     const int tid = threadIdx.x, B = blockDim.x;
     const int T = args.T;
@@ -140,7 +145,9 @@ __global__ void __launch_bounds__(128, 4) filter_kernel_global(const FilterArgs 
         uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
         for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
     }
-    load_zig_table(sh.zig, args.zig);
+    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
+    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
+    if (args.fast) load_fast_zig(fs, args.zig);
     if (tid == 0) sh.zig_g = args.zig;
     unsigned char *arrays = slabs + static_cast<size_t>(blockIdx.x) * slab_bytes;
     const int64_t F = args.M * T;
@@ -172,14 +179,17 @@ __global__ void __launch_bounds__(128, 4) filter_kernel_global(const FilterArgs 
         job.acc = args.acc ? args.acc + mrow : nullptr;
         job.reject_below = args.reject_below;
         job.slack = args.slack;
-        run_filter<RM, UM>(job, sh, arrays);
+        run_filter<RM, UM>(job, sh, args.fast != 0, fs, cols, arrays);
     }
 }
 
 template <int RM, int UM>
 int launch_tier_global(const FilterArgs &a, int B, unsigned char *slabs, size_t slab_bytes,
                        int grid, cudaStream_t s) {
-    filter_kernel_global<RM, UM><<<grid, B, 0, s>>>(a, slabs, slab_bytes);
+    const cudaError_t e = static_cast<cudaError_t>(
+        raise_smem_limit(reinterpret_cast<const void *>(filter_kernel_global<RM, UM>)));
+    if (e != cudaSuccess) return e;
+    filter_kernel_global<RM, UM><<<grid, B, a.fast, s>>>(a, slabs, slab_bytes);
     return cudaGetLastError();
 }
 
@@ -396,13 +406,28 @@ int reaction_tier(int R) {
 
 int global_grid(int sms) { return sms * 2; }
 
-size_t filter_static_smem() { return sizeof(SharedHead) + 2048; }
+size_t filter_static_smem() { return 30104; }
 
-int launch_filter(const FilterArgs &a, int B, double *loglik, uint8_t *status, void *stream,
+// Bytes of the fast path's tables and columns ahead of `population` bytes of
+// dynamic shared memory, or 0 when both do not fit a block together.
+int fast_smem(int U, int B, size_t population) {
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return 0;
+    const size_t f = (fast_smem_bytes(U, B) + 15) & ~static_cast<size_t>(15);
+    return f + population + sizeof(SharedHead) + 512 <= static_cast<size_t>(optin) ? static_cast<int>(f) : 0;
+}
+
+int launch_filter(const FilterArgs &args, int B, double *loglik, uint8_t *status, void *stream,
                   unsigned char *slabs, size_t slab_bytes, int grid) {
-    if (a.M == 0) return cudaSuccess;
+    if (args.M == 0) return cudaSuccess;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t smem = filter_smem_bytes(a.N, a.net.U, a.dg_f != nullptr);
+    FilterArgs a = args;
+    size_t smem = filter_smem_bytes(a.N, a.net.U, a.dg_f != nullptr);
+    if (a.cluster > 1) smem = cluster_smem_bytes(a.N, a.cluster, a.net.U, a.dg_f != nullptr);
+    a.fast = fast_smem(a.net.U, B, slabs ? 0 : smem);
+    smem += a.fast;
     int e;
     const bool small_u = a.net.U <= 4, tiny_u = a.net.U <= 2;
     if (slabs) {
@@ -417,7 +442,7 @@ int launch_filter(const FilterArgs &a, int B, double *loglik, uint8_t *status, v
         }
     } else if (a.cluster > 1) {
         const int C = a.cluster;
-        const size_t cs = cluster_smem_bytes(a.N, C, a.net.U, a.dg_f != nullptr);
+        const size_t cs = smem;
         switch (reaction_tier(a.net.R)) {
             case 4: e = tiny_u ? launch_tier_cluster<4, 2>(a, B, cs, C, s)
                     : small_u ? launch_tier_cluster<4, 4>(a, B, cs, C, s)
@@ -477,6 +502,20 @@ static void build_zig_table(ZigTab &t) {
         L.lo = f - m;
         L.hi = f + m;
         L.slope = i == 0 ? 0.0 : L.df / (t.x[i] - t.x[i + 1]);
+    }
+    for (int i = 0; i < kZigLayers; ++i) {
+        const float hi = static_cast<float>(t.x[i]);
+        t.fast_hi[i] = std::ldexp(hi, -24);
+        t.fast_lo[i] = std::ldexp(static_cast<float>(t.x[i] - static_cast<double>(hi)), -24);
+        // the product is monotone in u, so the test of the largest u with these
+        // upper 16 bits decides for all of them
+        int n = static_cast<int>(t.x[i + 1] / t.x[i] * 65536.0) + 1;
+        auto passes = [&](int top) {
+            const uint64_t uv = (static_cast<uint64_t>(top) << 37) - 1;
+            return std::ldexp(static_cast<double>(uv), -53) * t.x[i] < t.x[i + 1];
+        };
+        while (n > 0 && !passes(n)) --n;
+        t.fast_t[i] = static_cast<uint16_t>(std::max(0, std::min(n, 65536) - 16));
     }
 }
 

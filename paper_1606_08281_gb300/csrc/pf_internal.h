@@ -65,6 +65,7 @@ struct FilterArgs {
     double slack;               // upper bound of one per-time-point log increment, >= 0
     const ZigTab *zig;          // device copy of the exponential ziggurat table
     int32_t cluster;            // > 1: each filter split over a cluster of this many blocks
+    int32_t fast;               // bytes of shared memory of the SSA without FP64 (0: not used)
 };
 
 // Bytes of the particle population of one filter: N (8 + 4U + 4) bytes, plus
@@ -94,9 +95,13 @@ int raise_smem_limit(const void *kernel);
 // Resident blocks for the global-memory variant on a GPU with `sms` SMs.
 int global_grid(int sms);
 
-// Static shared memory of a filter block (its tables) plus a safety margin:
-// a population fits on chip when population + this <= the opt-in maximum.
+// What the on-chip limit counts for a block's tables: a population fits on
+// chip when population + this <= the opt-in maximum.
 size_t filter_static_smem();
+
+// Bytes of shared memory for the SSA without FP64 ahead of a population of the
+// given size (0: the two do not fit together, and the FP64 path runs).
+int fast_smem(int U, int block_threads, size_t population);
 
 // p[0..n) = value on `stream`.
 int launch_fill(double *p, int64_t n, double value, void *stream);

@@ -45,6 +45,11 @@ struct ZigLayer {
 struct ZigTab {
     double x[kZigLayers + 1];
     ZigLayer layer[kZigLayers];
+    // for the path without FP64 (ssa_fast.cuh): x_i 2^-24 as a sum of two
+    // floats, and the largest t such that every draw whose first word's upper
+    // 16 bits lie in 16 .. 15 + t passes the layer's test
+    float fast_hi[kZigLayers], fast_lo[kZigLayers];
+    uint16_t fast_t[kZigLayers];
 };
 
 // The shared-memory part: the layer edges the fast path reads.
