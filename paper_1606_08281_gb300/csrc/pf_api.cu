@@ -188,6 +188,9 @@ using pf::cuda_fail;
 using pf::build_tables;
 using pf::check_count_range;
 
+// Threads per filter block for n particles on it.
+int default_block(int n) { return std::min(n >= 512 ? 256 : 128, (n + 31) / 32 * 32); }
+
 struct DevBuf {
     void *p = nullptr;
     cudaStream_t s = nullptr;
@@ -257,8 +260,8 @@ int pf_loglik(const pf_network *net, const double *thetas, int64_t M, int32_t d,
     if (CB > 1 && N - (CB - 1) * Nb < 1)
         return fail(PF_EINVAL, "n_particles %d leaves a block of the %d-block cluster empty", N, CB);
     int B = o.block_threads;
-    if (B == 0) B = std::min(128, ((Nb + 31) / 32) * 32);
-    if (B < 32 || B > 128 || (B % 32)) return fail(PF_EINVAL, "block_threads %d must be a multiple of 32 in 32..128", B);
+    if (B == 0) B = default_block(Nb);
+    else if (B < 32 || B > 128 || (B % 32)) return fail(PF_EINVAL, "block_threads %d must be a multiple of 32 in 32..128", B);
     {
         int ze = 0;
         a.zig = pf::zig_table_device(&ze);
@@ -476,7 +479,7 @@ extern "C" int pf_loglik_noalloc(const pf_network *net, const double *thetas, in
         a.zig = pf::zig_table_device(&ze);
         if (!a.zig) return cuda_fail(ze, "ziggurat table");
     }
-    const int B = std::min(128, ((N + 31) / 32) * 32);
+    const int B = default_block(N);
     const size_t smem = pf::filter_smem_bytes(N, a.net.U, false);
     int dev = 0, smem_max = 0;
     PF_CUDA(cudaGetDevice(&dev), "cudaGetDevice");

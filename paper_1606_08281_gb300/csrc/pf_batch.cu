@@ -110,21 +110,18 @@ template <int RM, int UM, bool GLOBAL>
 __global__ void __launch_bounds__(kBlock, 4)
 batch_kernel(const BatchHeader *hdr, const RequestDev *reqs, const uint64_t *items, int group,
              unsigned long long *counters, unsigned char *slab, size_t slab_bytes, double *ll_f,
-             uint8_t *st_f, unsigned long long *ev_f, const ZigTab *zig, int grab, int fast) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SharedHead sh;
+             uint8_t *st_f, unsigned long long *ev_f, const ZigTab *zig, int grab, int offset) {
+    SharedHead &sh = block_head();
     __shared__ RequestDev rq;
     __shared__ unsigned long long cur;
     __shared__ uint64_t item;
     __shared__ const ProblemDev *loaded;
-    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
-    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
-    if (fast) load_fast_zig(fs, zig);
+    load_fast_zig(zig);
     if (threadIdx.x == 0) sh.zig_g = zig;
     if (threadIdx.x == 0) loaded = nullptr;
     const long long begin = hdr->group_begin[group];
     const unsigned long long count = static_cast<unsigned long long>(hdr->group_count[group]);
-    unsigned char *arrays = GLOBAL ? slab + static_cast<size_t>(blockIdx.x) * slab_bytes : smem + fast;
+    unsigned char *arrays = GLOBAL ? slab + static_cast<size_t>(blockIdx.x) * slab_bytes : g_smem + offset;
     unsigned long long base = 0;
     int left = 0;
     for (;;) {
@@ -169,7 +166,7 @@ batch_kernel(const BatchHeader *hdr, const RequestDev *reqs, const uint64_t *ite
         job.acc = rq.acc ? rq.acc + row : nullptr;
         job.reject_below = rq.reject_below;
         job.slack = rq.slack;
-        run_filter<RM, UM>(job, sh, fast != 0, fs, cols, arrays);
+        run_filter<RM, UM>(job, sh, SeedKeys{static_cast<uint32_t>(rq.seed), static_cast<uint32_t>(rq.seed >> 32)}, true, arrays);
     }
 }
 
@@ -182,18 +179,15 @@ template <int RM, int UM>
 __global__ void __launch_bounds__(kBlock, 2)
 batch_kernel_cluster(const BatchHeader *hdr, const RequestDev *reqs, const uint64_t *items,
                      int group, unsigned long long *counters, double *ll_f, uint8_t *st_f,
-                     unsigned long long *ev_f, const ZigTab *zig, int grab, int fast) {
+                     unsigned long long *ev_f, const ZigTab *zig, int grab, int offset) {
     namespace cg = cooperative_groups;
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SharedHead sh;
+    SharedHead &sh = block_head();
     __shared__ RequestDev rq;
     __shared__ unsigned long long cur, taken;
     __shared__ const ProblemDev *loaded;
     cg::cluster_group cl = cg::this_cluster();
     const bool lead = cl.block_rank() == 0;
-    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
-    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
-    if (fast) load_fast_zig(fs, zig);
+    load_fast_zig(zig);
     if (threadIdx.x == 0) sh.zig_g = zig;
     if (threadIdx.x == 0) loaded = nullptr;
     const long long begin = hdr->group_begin[group];
@@ -247,7 +241,7 @@ batch_kernel_cluster(const BatchHeader *hdr, const RequestDev *reqs, const uint6
         job.acc = rq.acc ? rq.acc + row : nullptr;
         job.reject_below = rq.reject_below;
         job.slack = rq.slack;
-        run_filter_cluster<RM, UM>(job, sh, fast != 0, fs, cols, smem + fast);
+        run_filter_cluster<RM, UM>(job, sh, SeedKeys{static_cast<uint32_t>(rq.seed), static_cast<uint32_t>(rq.seed >> 32)}, true, g_smem + offset);
     }
 }
 
@@ -325,9 +319,10 @@ int tier_of(const NetTables &t) {
 // pf_loglik launch sized for them would.  Larger populations go to the slabs.
 constexpr int kSmallArenaBlocks = 4, kLargeArenaBlocks = 2;
 
-// Bytes of the SSA without FP64 ahead of a tier's population arena.
-size_t tier_fast_bytes(int tier, int threads) {
-    return (fast_smem_bytes(tier == 0 ? 4 : PF_MAX_SPECIES, threads) + 15) & ~size_t(15);
+// Shared memory ahead of a tier's population arena: the block's head and the
+// tables and columns of the SSA without FP64.
+size_t tier_head_bytes(int tier, int threads) {
+    return kHeadBytes + fast_smem_bytes(tier == 0 ? 4 : PF_MAX_SPECIES, threads);
 }
 
 size_t population_bytes(int N, int U) { return filter_smem_bytes(N, U, false); }
@@ -378,7 +373,7 @@ struct Slot {
     unsigned char *slab[kGroups] = {};
     int grid[kGroups] = {};
     size_t smem[kGroups] = {};
-    int fast[kGroups] = {};             // of which the SSA without FP64 has these
+    int head[kGroups] = {};             // of which those ahead of the population
     std::vector<int64_t> ids;   // requests in flight on this slot
     bool busy = false;
     std::atomic<bool> finished{false};
@@ -467,7 +462,7 @@ int size_arenas(pf_ctx *ctx) {
         const cudaError_t e = static_cast<cudaError_t>(pf::raise_smem_limit(k));
         if (e != cudaSuccess) return pf::cuda_fail(e, "smem attribute");
         size_t small = 0, large = 0;
-        const size_t fast = tier_fast_bytes(t, ctx->block_threads[t]);
+        const size_t head = tier_head_bytes(t, ctx->block_threads[t]);
         CTX_CUDA(cudaOccupancyAvailableDynamicSMemPerBlock(&small, group_kernel(t, false),
                                                            t == 0 ? kSmallArenaBlocks : kSmallArenaBlocks - 1,
                                                            ctx->block_threads[t]),
@@ -475,8 +470,8 @@ int size_arenas(pf_ctx *ctx) {
         CTX_CUDA(cudaOccupancyAvailableDynamicSMemPerBlock(&large, group_kernel(t, false), kLargeArenaBlocks,
                                                            ctx->block_threads[t]),
                  "arena size");
-        ctx->arena[t][0] = (std::max(small, fast) - fast) & ~size_t(15);
-        ctx->arena[t][1] = (std::max(std::max(small, large), fast) - fast) & ~size_t(15);
+        ctx->arena[t][0] = (std::max(small, head) - head) & ~size_t(15);
+        ctx->arena[t][1] = (std::max(std::max(small, large), head) - head) & ~size_t(15);
     }
     return PF_OK;
 }
@@ -505,8 +500,8 @@ int init_slot(pf_ctx *ctx, int si) {
         const int B = ctx->block_threads[tier];
         if (kind == 2) {       // split filters: clusters of ctx->cluster blocks
             ClusterKernel ck = cluster_kernel(tier);
-            s.fast[g] = static_cast<int>(tier_fast_bytes(tier, B));
-            s.smem[g] = kClusterArena + s.fast[g];
+            s.head[g] = static_cast<int>(tier_head_bytes(tier, B));
+            s.smem[g] = kClusterArena + s.head[g];
             CTX_CUDA(static_cast<cudaError_t>(pf::raise_smem_limit(reinterpret_cast<const void *>(ck))),
                      "smem attribute");
             CTX_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeNonPortableClusterSizeAllowed, 1),
@@ -528,8 +523,8 @@ int init_slot(pf_ctx *ctx, int si) {
         } else {
             const bool global = kind == 1;
             BatchKernel k = group_kernel(tier, global);
-            s.fast[g] = static_cast<int>(tier_fast_bytes(tier, B));
-            s.smem[g] = s.fast[g] + (global ? 0 : ctx->arena[tier][kind == 3 ? 1 : 0]);
+            s.head[g] = static_cast<int>(tier_head_bytes(tier, B));
+            s.smem[g] = s.head[g] + (global ? 0 : ctx->arena[tier][kind == 3 ? 1 : 0]);
             CTX_CUDA(static_cast<cudaError_t>(pf::raise_smem_limit(reinterpret_cast<const void *>(k))),
                      "smem attribute");
             int occ = 0;
@@ -573,12 +568,12 @@ int init_slot(pf_ctx *ctx, int si) {
                                                       static_cast<const RequestDev *>(s.req_d),
                                                       static_cast<const uint64_t *>(s.items_d), g,
                                                       s.counters, s.ll_f, s.st_f, s.ev_f, zig,
-                                                      ctx->grab, s.fast[g]);
+                                                      ctx->grab, s.head[g]);
             if (le == cudaSuccess) le = e1;
         } else {
             group_kernel(tier, kind == 1)<<<s.grid[g], B, s.smem[g], s.side[g]>>>(
                 s.hdr_d, s.req_d, s.items_d, g, s.counters, s.slab[g], ctx->slab_bytes, s.ll_f,
-                s.st_f, s.ev_f, zig, ctx->grab, s.fast[g]);
+                s.st_f, s.ev_f, zig, ctx->grab, s.head[g]);
         }
         cudaEventRecord(s.join[g], s.side[g]);
         cudaStreamWaitEvent(s.stream, s.join[g], 0);

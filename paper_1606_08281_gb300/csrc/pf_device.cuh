@@ -49,12 +49,13 @@ constexpr int kMaxCluster = 8;     // blocks of a cluster that share one filter
 struct SharedHead {
     NetTables net;
     double rate[PF_MAX_REACTIONS];   // theta[rate_col[r]] of this filter's row
-    double red_d[kMaxWarps];
     unsigned long long red_u[kMaxWarps];
-    double bcast_d;
+    unsigned long long sum_lo[kMaxWarps], sum_hi[kMaxWarps];   // weight_sum's warp totals
     unsigned long long u_off;
     double ll;
     double lognorm;
+    double log_n;                      // log of the particle count
+    double pend_e[32], pend_s[32];     // emax and s of intervals not yet in ll
     int status;
     int valid;
     int pool_next;
@@ -64,11 +65,14 @@ struct SharedHead {
     double rem_t[2][kMaxRemnants];       // its time
     double inv_sigma[PF_MAX_OBS_DIM];  // 1 / sigma_p, correctly rounded
     const ZigTab *zig_g;      // the ziggurat table (global memory)
-    // exchange slot of a filter split over a thread-block cluster: each
-    // block's share, read by the others through distributed shared memory
-    double cx_lmax, cx_lsum;
-    unsigned long long cx_qtot, cx_fired, cx_dig;
-    int cx_status, cx_reject;
+    // a filter split over a thread-block cluster: entry r of the *_in arrays is
+    // block r's share, which it stores into every block's shared memory before
+    // the barrier (reads after it are local); the rest is read remotely
+    double cx_max_in[kMaxCluster], cx_sum_in[kMaxCluster];
+    unsigned long long cx_q_in[kMaxCluster];
+    int cx_st_in[kMaxCluster];
+    unsigned long long cx_fired, cx_dig;
+    int cx_reject;
     unsigned long long cx_cum[kMaxCluster];  // cumulative integer-weight totals per block
 };
 
@@ -440,13 +444,13 @@ __device__ __noinline__ void ssa_interval(SharedHead &sh, int *xs, int Np, int N
 }
 
 // One interval's simulation by the whole block; `redo` is scratch for N slots.
-template <int RM, int UM>
-__device__ __forceinline__ void simulate(SharedHead &sh, bool fast, FastShared &fs, int *cols, int *xs,
-                                         int Np, int N, int *redo, double t_prev, double t_end,
-                                         uint32_t key0, uint32_t key1, uint32_t lane, uint32_t mrow,
-                                         uint64_t budget, unsigned long long &fired, uint32_t j0) {
+template <int RM, int UM, class Keys>
+__device__ __forceinline__ void simulate(SharedHead &sh, bool fast, int *xs, int Np, int N, int *redo,
+                                         double t_prev, double t_end, const Keys &keys, uint32_t lane,
+                                         uint32_t mrow, uint64_t budget, unsigned long long &fired, uint32_t j0) {
+    const uint32_t key0 = keys.k0(0), key1 = keys.k1(0);
     const int tid = threadIdx.x;
-    if (fast) fast = fast_interval(fs, sh.net, sh.rate, xs, Np, N, t_prev, t_end, budget);
+    if (fast) fast = fast_interval(xs, Np, N, t_prev, t_end, budget);
     if (tid == 0) {
         sh.pool_next = fast ? static_cast<int>(blockDim.x) : 0;
         sh.rem_n[0] = 0;
@@ -457,9 +461,9 @@ __device__ __forceinline__ void simulate(SharedHead &sh, bool fast, FastShared &
         ssa_interval<RM, UM>(sh, xs, Np, N, nullptr, t_prev, t_end, key0, key1, lane, mrow, budget, fired, j0);
         return;
     }
-    ssa_fast<RM>(sh, fs, cols, xs, Np, N, key0, key1, lane, mrow, budget, fired, j0, redo);
+    fired += ssa_fast<RM, UM>(xs, Np, N, keys, lane, mrow, static_cast<uint32_t>(budget), j0, redo);
     __syncthreads();
-    const int again = fs.n_exact;
+    const int again = block_fast().n_exact;
     if (again > 0) {
         if (tid == 0) {
             sh.pool_next = 0;
@@ -505,20 +509,36 @@ __device__ __forceinline__ uint64_t slot_digest(uint32_t k, uint32_t j, uint32_t
     return slot_digest_at(k, j, anc, xs, Np, U, static_cast<int>(j));
 }
 
-// Block-wide reductions (every thread receives the result).
-__device__ __forceinline__ double block_max(double v, SharedHead &sh) {
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
+// Signed integers in the order of the doubles (NaN excluded), and back.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ static_cast<long long>(static_cast<unsigned long long>(b >> 63) >> 1);
+}
+__device__ __forceinline__ double order_value(long long k) {
+    return __longlong_as_double(k ^ static_cast<long long>(static_cast<unsigned long long>(k >> 63) >> 1));
+}
+
+// Warp-wide maximum of keys: the upper words', then the lower words' among them.
+__device__ __forceinline__ long long warp_max_key(long long k) {
+    const int hi = static_cast<int>(k >> 32);
+    const int mh = __reduce_max_sync(kFull, hi);
+    const unsigned ml = __reduce_max_sync(kFull, hi == mh ? static_cast<unsigned>(k) : 0u);
+    return (static_cast<long long>(mh) << 32) | ml;
+}
+
+// Block-wide maximum of order_key()s (every thread receives the value).  On
+// integers: an FP64 maximum would put its compares on the FP64 pipe.
+__device__ __forceinline__ double block_max(long long key, SharedHead &sh) {
+    key = warp_max_key(key);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (lane == 0) sh.red_u[warp] = static_cast<unsigned long long>(key);
     __syncthreads();
-    if (lane == 0) sh.red_d[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        double x = lane < nw ? sh.red_d[lane] : -INFINITY;
-        for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(kFull, x, o));
-        if (lane == 0) sh.bcast_d = x;
+    for (int w = 0; w < nw; ++w) {
+        const long long o = static_cast<long long>(sh.red_u[w]);
+        key = o > key ? o : key;
     }
     __syncthreads();
-    return sh.bcast_d;
+    return order_value(key);
 }
 
 __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v, SharedHead &sh) {
@@ -566,62 +586,90 @@ __device__ inline void block_scan_u64(unsigned long long *q, int N, SharedHead &
 }
 
 
-// The weights' sum s = sum_j exp(e_j - emax) over the n particles of wbuf,
-// in an order that does not depend on the block size: the particles form
-// chunks of 32 consecutive slots, each summed by a butterfly over a warp's
-// lanes; lane l of warp 0 then adds the chunk sums l, l + 32, ... in order,
-// and a last butterfly adds the lanes.  The chunk sums are kept in `spare`
-// (int [n], free during this step) as pairs of 32-bit words; one chunk needs
-// no storage.  The same exp() values give the integer weights of the next
-// resampling, written over the log-weights (wbuf and qbuf alias); with a
-// state-dependent variance those come from the log-weights rounded to
-// multiples of 2^-20 (grid20) instead.  Every thread receives s.
-__device__ __forceinline__ double weight_sum(double *wbuf, unsigned long long *qbuf, int *spare,
-                                             int n, double emax, bool svar, SharedHead &sh) {
+static __device__ __noinline__ unsigned long long weight_call(double a) {
+    return __double2ull_rz(__dmul_rn(exp(a), 4294967296.0));
+}
+
+// The integer weight floor(2^32 exp(a)), a <= 0, and exp(a) 2^62.  exp_neg_fixed
+// and exp() lie within 2^-51.9 of each other; where an integer lies in between,
+// exp() decides (1 in 2^18), so the weight is floor(2^32 exp(a)) of the FP64
+// function.
+__device__ __forceinline__ uint64_t weight_of(double a, const uint64_t *table, unsigned long long &q) {
+    const uint64_t V = exp_neg_fixed(a, table);
+    const uint64_t up = (V + 2048u) >> 30, down = (V - (V < 2048u ? V : 2048u)) >> 30;
+    q = V >> 30;
+    if (up != down && __double_as_longlong(a) << 1 != 0) q = weight_call(a);
+    return V;
+}
+
+static __device__ __noinline__ unsigned long long grid_weight(double e, double gmax, const uint64_t *table) {
+    unsigned long long q;
+    weight_of(__dsub_rn(grid20(e), gmax), table, q);
+    return q;
+}
+
+// The weights' sum s = sum_j exp(e_j - emax) over the n particles of wbuf, as
+// an exact sum of 62-bit fixed-point values (each within 2^-57 relative plus
+// 2^-61 of exp; an integer sum has no order, so s does not depend on the block
+// size), and the integer weights of the next resampling, written over the
+// log-weights (wbuf and qbuf alias).  With a state-dependent variance those come
+// from the log-weights rounded to multiples of 2^-20 (grid20).  A NaN
+// log-weight makes s NaN, and its integer weight is what exp() gives.  Every
+// thread receives s.  Of 40 FP64 instructions per particle 7 remain (the
+// log-weight and e - emax); what is run a few times per interval is bound by
+// instruction fetch, so the rare parts are out of line (telegraph, 4096 filters
+// of 200 particles and 25 times: 3.62 ms with them inline, 2.85 ms).
+__device__ __forceinline__ double weight_sum(double *wbuf, unsigned long long *qbuf, int n, double emax,
+                                             bool svar, SharedHead &sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int nchunk = (n + 31) >> 5;
-    const double gmax = grid20(emax);
-    double own = 0.0;    // warp 0, one chunk: the whole sum
-    for (int c = warp; c < nchunk; c += nw) {
-        const int j = (c << 5) + lane;
-        double v = 0.0;
-        if (j < n) {
-            const double e = wbuf[j];
-            v = exp(__dsub_rn(e, emax));
-            const double vq = svar ? exp(__dsub_rn(grid20(e), gmax)) : v;
-            qbuf[j] = __double2ull_rz(__dmul_rn(vq, 4294967296.0));
+    const uint64_t *table = sh.zig_g->exp_t;
+    const double gmax = svar ? grid20(emax) : 0.0;
+    unsigned long long lo = 0, hi = 0;
+    bool nan = false;
+    for (int j = tid; j < n; j += blockDim.x) {
+        const double e = wbuf[j], a = __dsub_rn(e, emax);
+        unsigned long long q;
+        uint64_t V = weight_of(a, table, q);
+        if ((__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) > 0x7FF0000000000000ll) {
+            nan = true;
+            q = __double2ull_rz(a);
+        } else if (svar) {
+            q = grid_weight(e, gmax, table);
         }
-        for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
-        if (nchunk == 1) {
-            own = v;
-        } else if (lane == 0) {
-            const long long b = __double_as_longlong(v);
-            spare[2 * c] = static_cast<int>(b);
-            spare[2 * c + 1] = static_cast<int>(b >> 32);
-        }
+        qbuf[j] = q;
+        lo += V & 0xFFFFFFFFull;
+        hi += V >> 32;
+    }
+    // three 24-bit limbs per lane, added over the warp
+    hi += lo >> 32;                                     // (hi, low word of lo)
+    const unsigned l0 = static_cast<unsigned>(lo) & 0xFFFFFFu;
+    const unsigned l1 = static_cast<unsigned>(((hi << 8) | (static_cast<unsigned>(lo) >> 24)) & 0xFFFFFFu);
+    const unsigned l2 = static_cast<unsigned>(hi >> 16);
+    const unsigned s0 = __reduce_add_sync(kFull, l0), s1 = __reduce_add_sync(kFull, l1);
+    const unsigned s2 = __reduce_add_sync(kFull, l2);
+    nan = __any_sync(kFull, nan);
+    if (lane == 0) {
+        sh.sum_lo[warp] = static_cast<unsigned long long>(s0) + (static_cast<unsigned long long>(s1) << 24);
+        sh.sum_hi[warp] = static_cast<unsigned long long>(s2) | (nan ? 1ull << 63 : 0ull);
     }
     __syncthreads();
-    if (warp == 0) {
-        double v = own;
-        if (nchunk > 1) {
-            v = 0.0;
-            for (int c = lane; c < nchunk; c += 32) {
-                const long long b = (static_cast<long long>(spare[2 * c + 1]) << 32) |
-                                    static_cast<unsigned int>(spare[2 * c]);
-                v = __dadd_rn(v, __longlong_as_double(b));
-            }
-            for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(kFull, v, o));
-        }
-        if (lane == 0) sh.bcast_d = v;
+    unsigned long long a0 = 0, a1 = 0;
+    for (int w = 0; w < nw; ++w) {
+        const unsigned long long h = sh.sum_hi[w];
+        nan = nan || (h >> 63) != 0;
+        a0 += sh.sum_lo[w];
+        a1 += h & ~(1ull << 63);
     }
-    __syncthreads();
-    return sh.bcast_d;
+    a1 += a0 >> 48;                                     // in units of 2^-14
+    a0 &= (1ull << 48) - 1ull;                          // in units of 2^-62
+    if (nan) return __longlong_as_double(0x7FF8000000000000ll);
+    return __fma_rn(static_cast<double>(a1), 1.0 / 16384.0, __dmul_rn(static_cast<double>(a0), 1.0 / 4611686018427387904.0));
 }
 
 // Per-filter set-up by the whole block: the theta row's validity (sh.valid),
 // the Gaussian normaliser, 1 / sigma_p and the reaction rates; ends with a
 // __syncthreads().
-__device__ __forceinline__ void filter_setup(const double *theta, SharedHead &sh) {
+__device__ __forceinline__ void filter_setup(const double *theta, SharedHead &sh, bool fast, int N) {
     const int tid = threadIdx.x;
     const int d = sh.net.d, R = sh.net.R, P = sh.net.P;
     if (tid == 0) {
@@ -638,11 +686,46 @@ __device__ __forceinline__ void filter_setup(const double *theta, SharedHead &sh
         double ln = 0.0;
         if (!sh.net.obs_state_var)
             for (int p = 0; p < P; ++p) ln = __dadd_rn(ln, log(sh.net.sigma[p]));
+        sh.log_n = log(static_cast<double>(N));
         sh.lognorm = __dadd_rn(ln, __dmul_rn(0.5 * static_cast<double>(P), log(2.0 * M_PI)));
         for (int p = 0; p < P; ++p) sh.inv_sigma[p] = __ddiv_rn(1.0, sh.net.sigma[p]);
     }
-    if (tid < R) sh.rate[tid] = reaction_rate(sh.net, theta, tid);
+    if (fast) {
+        fast_network();
+        __syncthreads();
+    }
+    for (int r = tid; r < R; r += blockDim.x) {
+        const double rate = reaction_rate(sh.net, theta, r);
+        sh.rate[r] = rate;
+        if (fast) fast_rate(r, rate);
+    }
     __syncthreads();
+}
+
+// Intervals' increments log p(y_k | y_<k) ~ log((1/N) sum_j l_j) are added to
+// sh.ll in order by warp 0, 32 of them at a time: a logarithm is 28 dependent
+// FP64 instructions of 63 cycles, and 32 lanes take as long as one.
+__device__ __forceinline__ double increment_of(const SharedHead &sh, double emax, double s) {
+    double inc = __dadd_rn(emax, log(s));
+    inc = __dsub_rn(inc, sh.log_n);
+    return __dsub_rn(inc, sh.lognorm);
+}
+__device__ __forceinline__ void flush_increments(SharedHead &sh, int n) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    const double inc = lane < n ? increment_of(sh, sh.pend_e[lane], sh.pend_s[lane]) : 0.0;
+    double ll = sh.ll;
+    for (int i = 0; i < n; ++i) ll = __dadd_rn(ll, __shfl_sync(kFull, inc, i));
+    __syncwarp();
+    if (lane == 0) sh.ll = ll;
+}
+// Warp 0, after interval k of K: keeps its (emax, s), or adds all that are kept.
+__device__ __forceinline__ void keep_increment(SharedHead &sh, int k, int K, double emax, double s) {
+    if (threadIdx.x == 0) {
+        sh.pend_e[k & 31] = emax;
+        sh.pend_s[k & 31] = s;
+    }
+    if ((k & 31) == 31 || k == K - 1) flush_increments(sh, (k & 31) + 1);
 }
 
 // Initial state of particle j (column jl of xs): x0, or each count uniform on
@@ -673,35 +756,60 @@ __device__ __forceinline__ void init_particle(const SharedHead &sh, int *xs, int
     }
 }
 
+// v / 2 exactly for v >= 0, on the integer pipe where the result is normal.
+__device__ __forceinline__ double half_of(double v) {
+    const long long b = __double_as_longlong(v);
+    const bool normal = b >= (2ll << 52) && b < (0x7FFll << 52);
+    return normal ? __longlong_as_double(b - (1ll << 52)) : __dmul_rn(0.5, v);
+}
+
+// offset + sum_u c_u x_u, added in species order.  Terms with a zero
+// coefficient add +-0 exactly and are skipped, as are a product with 1 and a sum
+// onto a zero offset (all warp-uniform tests on bits); counts convert to
+// double on the integer pipes.
+__device__ __forceinline__ double affine(double offset, const double *c, const int *xs, int Np, int U, int j) {
+    double mu = offset;
+    bool zero = !nonzero(offset);
+    for (int u = 0; u < U; ++u) {
+        if (!nonzero(c[u])) continue;
+        const double x = count32_to_double(xs[u * Np + j]);
+        const double p = __double_as_longlong(c[u]) == 0x3FF0000000000000ll ? x : __dmul_rn(c[u], x);
+        mu = zero ? p : __dadd_rn(mu, p);
+        zero = false;
+    }
+    return mu;
+}
+
 // Gaussian log-weight exponent of the particle in column j of xs:
 // e_j = -1/2 sum_p ((y_p - mu_p) / sigma_p)^2 with mu_p = offset_p + (C x_j)_p;
 // with a state-dependent variance v_p = sigma_p^2 + sum_u V_pu x_u,
-// e_j = -1/2 sum_p ((y_p - mu_p)^2 / v_p + log v_p).  Terms with a zero
-// coefficient add +-0 exactly and are skipped (a warp-uniform test on the
-// coefficient's bits); counts convert to double on the integer pipes.
-__device__ __forceinline__ double log_weight(const SharedHead &sh, const int *xs, int Np, int j,
-                                             const double *yk, bool svar) {
+// e_j = -1/2 sum_p ((y_p - mu_p)^2 / v_p + log v_p) (out of line: the common
+// case's code, run once or a few times per interval, is bound by instruction
+// fetch).
+static __device__ __noinline__ double log_weight_svar(const SharedHead &sh, const int *xs, int Np, int j,
+                                                      const double *yk) {
     const int P = sh.net.P, U = sh.net.U;
     double acc = 0.0, lv = 0.0;
     for (int p = 0; p < P; ++p) {
-        double mu = sh.net.obs_offset[p];
-        for (int u = 0; u < U; ++u)
-            if (nonzero(sh.net.C[p][u]))
-                mu = __dadd_rn(mu, __dmul_rn(sh.net.C[p][u], count_to_double(xs[u * Np + j])));
-        if (svar) {
-            double v = __dmul_rn(sh.net.sigma[p], sh.net.sigma[p]);
-            for (int u = 0; u < U; ++u)
-                if (nonzero(sh.net.obs_var[p][u]))
-                    v = __dadd_rn(v, __dmul_rn(sh.net.obs_var[p][u], count_to_double(xs[u * Np + j])));
-            const double dv = __dsub_rn(yk[p], mu);
-            acc = __dadd_rn(acc, __ddiv_rn(__dmul_rn(dv, dv), v));
-            lv = __dadd_rn(lv, log(v));
-        } else {
-            const double z = div_by_recip(__dsub_rn(yk[p], mu), sh.net.sigma[p], sh.inv_sigma[p]);
-            acc = __dadd_rn(acc, __dmul_rn(z, z));
-        }
+        const double dv = __dsub_rn(yk[p], affine(sh.net.obs_offset[p], sh.net.C[p], xs, Np, U, j));
+        const double v = affine(__dmul_rn(sh.net.sigma[p], sh.net.sigma[p]), sh.net.obs_var[p], xs, Np, U, j);
+        acc = __dadd_rn(acc, __ddiv_rn(__dmul_rn(dv, dv), v));
+        lv = __dadd_rn(lv, log(v));
     }
-    return svar ? __dmul_rn(-0.5, __dadd_rn(acc, lv)) : __dmul_rn(-0.5, acc);
+    return __dmul_rn(-0.5, __dadd_rn(acc, lv));
+}
+__device__ __forceinline__ double log_weight(const SharedHead &sh, const int *xs, int Np, int j,
+                                             const double *yk, bool svar) {
+    if (svar) return log_weight_svar(sh, xs, Np, j, yk);
+    const int P = sh.net.P, U = sh.net.U;
+    double acc = 0.0;
+    for (int p = 0; p < P; ++p) {
+        const double dv = __dsub_rn(yk[p], affine(sh.net.obs_offset[p], sh.net.C[p], xs, Np, U, j));
+        const double z = div_by_recip(dv, sh.net.sigma[p], sh.inv_sigma[p]);
+        const double z2 = __dmul_rn(z, z);
+        acc = p == 0 ? z2 : __dadd_rn(acc, z2);
+    }
+    return -half_of(acc);
 }
 
 // One filter -- one (theta row, observed trajectory) pair -- through all K
@@ -734,14 +842,12 @@ struct FilterJob {
     double slack;
 };
 
-template <int RM, int UM>
-__device__ void run_filter(const FilterJob &job, SharedHead &sh, bool fast, FastShared &fs, int *cols,
-                           unsigned char *arrays) {
+template <int RM, int UM, class Keys>
+__device__ void run_filter(const FilterJob &job, SharedHead &sh, const Keys &keys, bool fast, unsigned char *arrays) {
     const int tid = threadIdx.x, B = blockDim.x;
     const int U = sh.net.U, P = sh.net.P;
     const int N = job.N, K = job.K;
-    if (fast) fast_network(fs, cols, sh.net);
-    filter_setup(job.theta, sh);
+    filter_setup(job.theta, sh, fast, N);
     if (!sh.valid) {
         if (tid == 0) {
             *job.ll_out = __longlong_as_double(0x7FF8000000000000ll);
@@ -843,7 +949,7 @@ __device__ void run_filter(const FilterJob &job, SharedHead &sh, bool fast, Fast
             // the pool hands out particle slots in index order (the refill
             // loop and the tail consolidation absorb their unequal costs;
             // sorting them heaviest first no longer paid for its two passes)
-            simulate<RM, UM>(sh, fast, fs, cols, xs, Np, N, order, t_prev, t_k, key0, key1, lane, m32,
+            simulate<RM, UM>(sh, fast, xs, Np, N, order, t_prev, t_k, keys, lane, m32,
                              job.budget, fired, 0u);
         }
         __syncthreads();
@@ -862,11 +968,11 @@ __device__ void run_filter(const FilterJob &job, SharedHead &sh, bool fast, Fast
         // Gaussian log-weight exponents (Supp. I, "Compute weights")
         const double *yk = job.y + static_cast<int64_t>(k) * P;
         const bool svar = sh.net.obs_state_var != 0;
-        double lmax = -INFINITY;
+        long long lmax = order_key(-INFINITY);
         for (int j = tid; j < N; j += B) {
             const double e = log_weight(sh, xs, Np, j, yk, svar);
             wbuf[j] = e;
-            lmax = fmax(lmax, e);
+            if (e == e) lmax = max(lmax, order_key(e));
         }
         const double emax = block_max(lmax, sh);
         if (!isfinite(emax)) {
@@ -875,17 +981,17 @@ __device__ void run_filter(const FilterJob &job, SharedHead &sh, bool fast, Fast
         }
         // p(y_k | y_<k) ~ (1/N) sum_j l_j  (Eq. likelihood approx.), in logs;
         // the same exp() values give the integer weights for the next resampling
-        const double s = weight_sum(wbuf, qbuf, order, N, emax, svar, sh);
-        if (tid == 0) {
-            double inc = __dadd_rn(emax, log(s));
-            inc = __dsub_rn(inc, log(static_cast<double>(N)));
-            inc = __dsub_rn(inc, sh.lognorm);
-            sh.ll = __dadd_rn(sh.ll, inc);
-            if (job.acc) {
+        const double s = weight_sum(wbuf, qbuf, N, emax, svar, sh);
+        if (job.acc) {
+            if (tid == 0) {
+                const double inc = increment_of(sh, emax, s);
+                sh.ll = __dadd_rn(sh.ll, inc);
                 const double add = __dsub_rn(inc, job.slack);
                 if (__dadd_rn(atomicAdd(job.acc, add), add) < job.reject_below)
                     sh.status = PF_ST_REJECTED;
             }
+        } else if (tid < 32) {
+            keep_increment(sh, k, K, emax, s);
         }
         if (want_ph) ph[2] += static_cast<unsigned long long>(clock64() - c_mark);
         t_prev = t_k;
@@ -939,9 +1045,8 @@ __host__ __device__ __forceinline__ size_t cluster_share_bytes(int N, int C, int
 // rank order).  Every decision to leave the loop is taken from exchanged
 // values after a cluster barrier, so all blocks pass the same barriers.
 // Requires n >= 1 in every block (N > (C - 1) ceil(N / C)); checked by the host.
-template <int RM, int UM>
-__device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fast, FastShared &fs,
-                                   int *cols, unsigned char *arrays) {
+template <int RM, int UM, class Keys>
+__device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, const Keys &keys, bool fast, unsigned char *arrays) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int C = static_cast<int>(cl.num_blocks());
@@ -952,8 +1057,7 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fa
     const int Np = (N + C - 1) / C;
     const int j0 = rank * Np;
     const int n = min(Np, N - j0);
-    if (fast) fast_network(fs, cols, sh.net);
-    filter_setup(job.theta, sh);
+    filter_setup(job.theta, sh, fast, N);
     if (!sh.valid) {           // the same row in every block: all leave here
         if (tid == 0 && rank == 0) {
             *job.ll_out = __longlong_as_double(0x7FF8000000000000ll);
@@ -988,6 +1092,8 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fa
             sh.cx_reject = *reinterpret_cast<volatile double *>(job.acc) < job.reject_below;
         cl.sync();
         if (*cl.map_shared_rank(&sh.cx_reject, 0)) status = PF_ST_REJECTED;
+    } else {
+        cl.sync();             // every block runs before another stores into its shared memory
     }
     const unsigned long long Nl = static_cast<unsigned long long>(N);
     for (int k = 0; k < K && status == PF_ST_OK; ++k) {
@@ -1030,7 +1136,7 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fa
 
         const double t_k = job.obs_times[k];
         if (t_k > t_prev) {
-            simulate<RM, UM>(sh, fast, fs, cols, xs, Np, n, order, t_prev, t_k, key0, key1, lane, m32,
+            simulate<RM, UM>(sh, fast, xs, Np, n, order, t_prev, t_k, keys, lane, m32,
                              job.budget, fired, static_cast<uint32_t>(j0));
         }
         __syncthreads();
@@ -1042,25 +1148,25 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fa
 
         const double *yk = job.y + static_cast<int64_t>(k) * P;
         const bool svar = sh.net.obs_state_var != 0;
-        double lmax = -INFINITY;
+        long long lmax = order_key(-INFINITY);
         for (int jl = tid; jl < n; jl += B) {
             const double e = log_weight(sh, xs, Np, jl, yk, svar);
             wbuf[jl] = e;
-            lmax = fmax(lmax, e);
+            if (e == e) lmax = max(lmax, order_key(e));
         }
         const double bmax = block_max(lmax, sh);
-        if (tid == 0) {
-            sh.cx_lmax = bmax;
-            sh.cx_status = sh.status;
+        if (tid < C) {
+            *cl.map_shared_rank(&sh.cx_max_in[rank], tid) = bmax;
+            *cl.map_shared_rank(&sh.cx_st_in[rank], tid) = sh.status;
         }
         cl.sync();   // A
-        double emax = -INFINITY;
+        long long kmax = order_key(-INFINITY);
         int st = PF_ST_OK;
         for (int r = 0; r < C; ++r) {
-            emax = fmax(emax, *cl.map_shared_rank(&sh.cx_lmax, r));
-            const int sr = *cl.map_shared_rank(&sh.cx_status, r);
-            if (st == PF_ST_OK) st = sr;
+            kmax = max(kmax, order_key(sh.cx_max_in[r]));
+            if (st == PF_ST_OK) st = sh.cx_st_in[r];
         }
+        const double emax = order_value(kmax);
         if (st != PF_ST_OK) {
             status = st;
             break;
@@ -1069,30 +1175,34 @@ __device__ void run_filter_cluster(const FilterJob &job, SharedHead &sh, bool fa
             status = PF_ST_NONFINITE;
             break;
         }
-        const double bsum = weight_sum(wbuf, qbuf, order, n, emax, svar, sh);
+        const double bsum = weight_sum(wbuf, qbuf, n, emax, svar, sh);
         block_scan_u64(qbuf, n, sh);
-        if (tid == 0) {
-            sh.cx_lsum = bsum;
-            sh.cx_qtot = qbuf[n - 1];
+        if (tid < C) {
+            *cl.map_shared_rank(&sh.cx_sum_in[rank], tid) = bsum;
+            *cl.map_shared_rank(&sh.cx_q_in[rank], tid) = qbuf[n - 1];
         }
         cl.sync();   // B
-        if (tid == 0) {
-            double s = 0.0;
-            unsigned long long run = 0;
-            for (int r = 0; r < C; ++r) {
-                s = __dadd_rn(s, *cl.map_shared_rank(&sh.cx_lsum, r));
-                run += *cl.map_shared_rank(&sh.cx_qtot, r);
-                sh.cx_cum[r] = run;
+        if (tid < 32) {
+            // cumulative totals of the blocks (a lane each), the sum in rank order
+            unsigned long long q = tid < C ? sh.cx_q_in[tid] : 0ull;
+            for (int o = 1; o < kMaxCluster; o <<= 1) {
+                const unsigned long long v = __shfl_up_sync(kFull, q, o);
+                if (tid >= o) q += v;
             }
+            if (tid < C) sh.cx_cum[tid] = q;
             if (rank == 0) {
-                double inc = __dadd_rn(emax, log(s));
-                inc = __dsub_rn(inc, log(static_cast<double>(N)));
-                inc = __dsub_rn(inc, sh.lognorm);
-                sh.ll = __dadd_rn(sh.ll, inc);
-                sh.cx_reject = 0;
+                double s = 0.0;
+                for (int r = 0; r < C; ++r) s = __dadd_rn(s, sh.cx_sum_in[r]);
                 if (job.acc) {
-                    const double add = __dsub_rn(inc, job.slack);
-                    sh.cx_reject = __dadd_rn(atomicAdd(job.acc, add), add) < job.reject_below;
+                    if (tid == 0) {
+                        const double inc = increment_of(sh, emax, s);
+                        sh.ll = __dadd_rn(sh.ll, inc);
+                        const double add = __dsub_rn(inc, job.slack);
+                        sh.cx_reject = __dadd_rn(atomicAdd(job.acc, add), add) < job.reject_below;
+                    }
+                } else {
+                    if (tid == 0) sh.cx_reject = 0;
+                    keep_increment(sh, k, K, emax, s);
                 }
             }
         }

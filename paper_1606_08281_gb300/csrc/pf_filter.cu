@@ -27,170 +27,24 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <mutex>
 #include <utility>
 #include <vector>
 
-#include "pf_device.cuh"
+#include "pf_filter.cuh"
 
 namespace pf {
 namespace {
 
 using namespace dev;
 
-// ------------------------------------------------------------------ kernels
-template <int RM, int UM>
-__global__ void __launch_bounds__(128, 4) filter_kernel(const FilterArgs args) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SharedHead sh;
-    const int tid = threadIdx.x, B = blockDim.x;
-    const int T = args.T;
-    const int64_t slot = blockIdx.x;
-    int64_t mrow = slot / T;
-    const int traj = static_cast<int>(slot - mrow * T);
-    if (args.row_order) mrow = args.row_order[mrow];
-    const int64_t f = mrow * T + traj;
-    {  // network tables -> shared memory
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(&args.net);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
-        for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
-    }
-    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
-    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
-    if (args.fast) load_fast_zig(fs, args.zig);
-    if (tid == 0) sh.zig_g = args.zig;
+template <int RM, int UM, int MT>
+__global__ void __launch_bounds__(MT, kMinBlocks<RM, MT>) filter_kernel(const __grid_constant__ FilterArgs args) {
+    load_head(args);
     __syncthreads();
-    FilterJob job;
-    job.theta = args.thetas + mrow * args.net.d;
-    job.obs_times = args.obs_times;
-    job.y = args.y + static_cast<int64_t>(traj) * args.K * args.net.P;
-    job.K = args.K;
-    job.N = args.N;
-    job.mrow = args.theta_ids ? args.theta_ids[mrow] : static_cast<uint32_t>(mrow);
-    job.traj = traj;
-    job.seed = args.seed;
-    job.budget = args.budget;
-    job.ll_out = args.ll_f + f;
-    job.st_out = args.st_f + f;
-    job.ev_out = reinterpret_cast<unsigned long long *>(args.ev_f) + f;
-    job.dg_out = args.dg_f ? reinterpret_cast<unsigned long long *>(args.dg_f) + f : nullptr;
-    job.fs_out = args.final_states ? args.final_states + f * static_cast<int64_t>(args.N) * args.net.U
-                                   : nullptr;
-    job.ph_out = args.phase_f ? reinterpret_cast<unsigned long long *>(args.phase_f) + 3 * f : nullptr;
-    job.acc = args.acc ? args.acc + mrow : nullptr;
-    job.reject_below = args.reject_below;
-    job.slack = args.slack;
-    run_filter<RM, UM>(job, sh, args.fast != 0, fs, cols, smem + args.fast);
-}
-
-// A filter split over the C blocks of a thread-block cluster (cluster size
-// set at launch): cluster c runs filter slot c, its blocks on C SMs.
-template <int RM, int UM>
-__global__ void __launch_bounds__(128, 4) filter_kernel_cluster(const FilterArgs args) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SharedHead sh;
-    const int tid = threadIdx.x, B = blockDim.x;
-    const int T = args.T;
-    const int64_t slot = blockIdx.x / cooperative_groups::this_cluster().num_blocks();
-    int64_t mrow = slot / T;
-    const int traj = static_cast<int>(slot - mrow * T);
-    if (args.row_order) mrow = args.row_order[mrow];
-    const int64_t f = mrow * T + traj;
-    {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(&args.net);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
-        for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
-    }
-    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
-    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
-    if (args.fast) load_fast_zig(fs, args.zig);
-    if (tid == 0) sh.zig_g = args.zig;
-    __syncthreads();
-    FilterJob job;
-    job.theta = args.thetas + mrow * args.net.d;
-    job.obs_times = args.obs_times;
-    job.y = args.y + static_cast<int64_t>(traj) * args.K * args.net.P;
-    job.K = args.K;
-    job.N = args.N;
-    job.mrow = args.theta_ids ? args.theta_ids[mrow] : static_cast<uint32_t>(mrow);
-    job.traj = traj;
-    job.seed = args.seed;
-    job.budget = args.budget;
-    job.ll_out = args.ll_f + f;
-    job.st_out = args.st_f + f;
-    job.ev_out = reinterpret_cast<unsigned long long *>(args.ev_f) + f;
-    job.dg_out = args.dg_f ? reinterpret_cast<unsigned long long *>(args.dg_f) + f : nullptr;
-    job.fs_out = args.final_states ? args.final_states + f * static_cast<int64_t>(args.N) * args.net.U
-                                   : nullptr;
-    job.ph_out = args.phase_f ? reinterpret_cast<unsigned long long *>(args.phase_f) + 3 * f : nullptr;
-    job.acc = args.acc ? args.acc + mrow : nullptr;
-    job.reject_below = args.reject_below;
-    job.slack = args.slack;
-    run_filter_cluster<RM, UM>(job, sh, args.fast != 0, fs, cols, smem + args.fast);
-}
-
-// Populations too large for shared memory: a grid of resident blocks walks
-// the filters (grid stride), each block keeping its population in its own slab
-// of global memory (N (16 + 8U) bytes), which stays in L1/L2 while it runs.
-template <int RM, int UM>
-__global__ void __launch_bounds__(128, 4) filter_kernel_global(const FilterArgs args,
-                                                               unsigned char *slabs,
-                                                               size_t slab_bytes) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SharedHead sh;
-    const int tid = threadIdx.x, B = blockDim.x;
-    const int T = args.T;
-    {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(&args.net);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.net);
-        for (int i = tid; i < static_cast<int>(sizeof(NetTables) / 4); i += B) dst[i] = src[i];
-    }
-    FastShared &fs = *reinterpret_cast<FastShared *>(smem);
-    int *cols = reinterpret_cast<int *>(smem + sizeof(FastShared));
-    if (args.fast) load_fast_zig(fs, args.zig);
-    if (tid == 0) sh.zig_g = args.zig;
-    unsigned char *arrays = slabs + static_cast<size_t>(blockIdx.x) * slab_bytes;
-    const int64_t F = args.M * T;
-    for (int64_t slot = blockIdx.x; slot < F; slot += gridDim.x) {
-        __syncthreads();
-        int64_t mrow = slot / T;
-        const int traj = static_cast<int>(slot - mrow * T);
-        if (args.row_order) mrow = args.row_order[mrow];
-        const int64_t f = mrow * T + traj;
-        FilterJob job;
-        job.theta = args.thetas + mrow * args.net.d;
-        job.obs_times = args.obs_times;
-        job.y = args.y + static_cast<int64_t>(traj) * args.K * args.net.P;
-        job.K = args.K;
-        job.N = args.N;
-        job.mrow = args.theta_ids ? args.theta_ids[mrow] : static_cast<uint32_t>(mrow);
-        job.traj = traj;
-        job.seed = args.seed;
-        job.budget = args.budget;
-        job.ll_out = args.ll_f + f;
-        job.st_out = args.st_f + f;
-        job.ev_out = reinterpret_cast<unsigned long long *>(args.ev_f) + f;
-        job.dg_out = args.dg_f ? reinterpret_cast<unsigned long long *>(args.dg_f) + f : nullptr;
-        job.fs_out = args.final_states
-                         ? args.final_states + f * static_cast<int64_t>(args.N) * args.net.U
-                         : nullptr;
-        job.ph_out = args.phase_f ? reinterpret_cast<unsigned long long *>(args.phase_f) + 3 * f
-                                  : nullptr;
-        job.acc = args.acc ? args.acc + mrow : nullptr;
-        job.reject_below = args.reject_below;
-        job.slack = args.slack;
-        run_filter<RM, UM>(job, sh, args.fast != 0, fs, cols, arrays);
-    }
-}
-
-template <int RM, int UM>
-int launch_tier_global(const FilterArgs &a, int B, unsigned char *slabs, size_t slab_bytes,
-                       int grid, cudaStream_t s) {
-    const cudaError_t e = static_cast<cudaError_t>(
-        raise_smem_limit(reinterpret_cast<const void *>(filter_kernel_global<RM, UM>)));
-    if (e != cudaSuccess) return e;
-    filter_kernel_global<RM, UM><<<grid, B, a.fast, s>>>(a, slabs, slab_bytes);
-    return cudaGetLastError();
+    run_filter<RM, UM>(filter_job(args, blockIdx.x), block_head(), ParamKeys{args.round_keys}, args.fast != 0,
+                       g_smem + kHeadBytes + args.fast);
 }
 
 // loglik[m] = sum over trajectories (in order) of the filter estimates (Supp. I).
@@ -328,39 +182,33 @@ __global__ void philox_kernel(const uint32_t *ctr, const uint32_t *key, uint32_t
     out[4 * i + 3] = w.w3;
 }
 
+// The instance for B threads: small networks have one for blocks of up to 128.
+template <int RM, int UM>
+auto filter_instance(int B) {
+    if constexpr (RM <= 8) return B <= 128 ? filter_kernel<RM, UM, 128> : filter_kernel<RM, UM, kMaxThreads>;
+    else return filter_kernel<RM, UM, kMaxThreads>;
+}
 template <int RM, int UM>
 int launch_tier(const FilterArgs &a, int B, size_t smem, cudaStream_t s) {
-    cudaError_t e = static_cast<cudaError_t>(
-        raise_smem_limit(reinterpret_cast<const void *>(filter_kernel<RM, UM>)));
+    const auto kernel = filter_instance<RM, UM>(B);
+    cudaError_t e = static_cast<cudaError_t>(raise_smem_limit(reinterpret_cast<const void *>(kernel)));
     if (e != cudaSuccess) return e;
     const int64_t F = a.M * a.T;
-    filter_kernel<RM, UM><<<static_cast<unsigned>(F), B, smem, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <int RM, int UM>
-int launch_tier_cluster(const FilterArgs &a, int B, size_t smem, int C, cudaStream_t s) {
-    cudaError_t e = static_cast<cudaError_t>(
-        raise_smem_limit(reinterpret_cast<const void *>(filter_kernel_cluster<RM, UM>)));
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(a.M * a.T * C));
-    cfg.blockDim = dim3(static_cast<unsigned>(B));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(C);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, filter_kernel_cluster<RM, UM>, a);
-    if (e != cudaSuccess) return e;
+    kernel<<<static_cast<unsigned>(F), B, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 }  // namespace
+
+static int launch_filter_plain(const FilterArgs &a, int B, size_t smem, cudaStream_t s) {
+    const bool small_u = a.net.U <= 4, tiny_u = a.net.U <= 2;
+    switch (reaction_tier(a.net.R)) {
+        case 4: return tiny_u ? launch_tier<4, 2>(a, B, smem, s) : small_u ? launch_tier<4, 4>(a, B, smem, s) : launch_tier<4, 0>(a, B, smem, s);
+        case 8: return small_u ? launch_tier<8, 4>(a, B, smem, s) : launch_tier<8, 0>(a, B, smem, s);
+        case 16: return launch_tier<16, 0>(a, B, smem, s);
+        default: return launch_tier<32, 0>(a, B, smem, s);
+    }
+}
 
 // The dynamic shared-memory limit of a kernel is a process-wide attribute.
 // It is raised once per kernel and device to the largest size a launch of it
@@ -415,8 +263,8 @@ int fast_smem(int U, int B, size_t population) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return 0;
-    const size_t f = (fast_smem_bytes(U, B) + 15) & ~static_cast<size_t>(15);
-    return f + population + sizeof(SharedHead) + 512 <= static_cast<size_t>(optin) ? static_cast<int>(f) : 0;
+    const size_t f = fast_smem_bytes(U, B);
+    return kHeadBytes + f + population + 512 <= static_cast<size_t>(optin) ? static_cast<int>(f) : 0;
 }
 
 int launch_filter(const FilterArgs &args, int B, double *loglik, uint8_t *status, void *stream,
@@ -427,38 +275,14 @@ int launch_filter(const FilterArgs &args, int B, double *loglik, uint8_t *status
     size_t smem = filter_smem_bytes(a.N, a.net.U, a.dg_f != nullptr);
     if (a.cluster > 1) smem = cluster_smem_bytes(a.N, a.cluster, a.net.U, a.dg_f != nullptr);
     a.fast = fast_smem(a.net.U, B, slabs ? 0 : smem);
-    smem += a.fast;
-    int e;
-    const bool small_u = a.net.U <= 4, tiny_u = a.net.U <= 2;
-    if (slabs) {
-        switch (reaction_tier(a.net.R)) {
-            case 4: e = tiny_u ? launch_tier_global<4, 2>(a, B, slabs, slab_bytes, grid, s)
-                    : small_u ? launch_tier_global<4, 4>(a, B, slabs, slab_bytes, grid, s)
-                              : launch_tier_global<4, 0>(a, B, slabs, slab_bytes, grid, s); break;
-            case 8: e = small_u ? launch_tier_global<8, 4>(a, B, slabs, slab_bytes, grid, s)
-                                : launch_tier_global<8, 0>(a, B, slabs, slab_bytes, grid, s); break;
-            case 16: e = launch_tier_global<16, 0>(a, B, slabs, slab_bytes, grid, s); break;
-            default: e = launch_tier_global<32, 0>(a, B, slabs, slab_bytes, grid, s); break;
-        }
-    } else if (a.cluster > 1) {
-        const int C = a.cluster;
-        const size_t cs = smem;
-        switch (reaction_tier(a.net.R)) {
-            case 4: e = tiny_u ? launch_tier_cluster<4, 2>(a, B, cs, C, s)
-                    : small_u ? launch_tier_cluster<4, 4>(a, B, cs, C, s)
-                              : launch_tier_cluster<4, 0>(a, B, cs, C, s); break;
-            case 8: e = small_u ? launch_tier_cluster<8, 4>(a, B, cs, C, s)
-                                : launch_tier_cluster<8, 0>(a, B, cs, C, s); break;
-            case 16: e = launch_tier_cluster<16, 0>(a, B, cs, C, s); break;
-            default: e = launch_tier_cluster<32, 0>(a, B, cs, C, s); break;
-        }
-    } else switch (reaction_tier(a.net.R)) {
-        case 4: e = tiny_u ? launch_tier<4, 2>(a, B, smem, s)
-                : small_u ? launch_tier<4, 4>(a, B, smem, s) : launch_tier<4, 0>(a, B, smem, s); break;
-        case 8: e = small_u ? launch_tier<8, 4>(a, B, smem, s) : launch_tier<8, 0>(a, B, smem, s); break;
-        case 16: e = launch_tier<16, 0>(a, B, smem, s); break;
-        default: e = launch_tier<32, 0>(a, B, smem, s); break;
+    for (uint32_t i = 0; i < 10; ++i) {
+        a.round_keys[i] = static_cast<uint32_t>(a.seed) + i * 0x9E3779B9u;
+        a.round_keys[10 + i] = static_cast<uint32_t>(a.seed >> 32) + i * 0xBB67AE85u;
     }
+    smem += kHeadBytes + a.fast;
+    const int e = slabs ? launch_filter_global(a, B, slabs, slab_bytes, grid, s)
+                  : a.cluster > 1 ? launch_filter_cluster(a, B, smem, s)
+                                  : launch_filter_plain(a, B, smem, s);
     if (e != cudaSuccess) return e;
     const int rb = 128;
     reduce_kernel<<<static_cast<unsigned>((a.M + rb - 1) / rb), rb, 0, s>>>(a.ll_f, a.st_f, a.M,
@@ -503,10 +327,16 @@ static void build_zig_table(ZigTab &t) {
         L.hi = f + m;
         L.slope = i == 0 ? 0.0 : L.df / (t.x[i] - t.x[i + 1]);
     }
+    for (int i = 0; i < kExpTable; ++i)
+        t.exp_t[i] = static_cast<uint64_t>(std::ldexp(std::exp(-i * 0.693147180559945309417232121458176568L / kExpTable), 63) + 0.5L);
     for (int i = 0; i < kZigLayers; ++i) {
         const float hi = static_cast<float>(t.x[i]);
         t.fast_hi[i] = std::ldexp(hi, -24);
-        t.fast_lo[i] = std::ldexp(static_cast<float>(t.x[i] - static_cast<double>(hi)), -24);
+        const float lo = std::ldexp(static_cast<float>(t.x[i] - static_cast<double>(hi)), -24);
+        uint32_t lo_bits;
+        memcpy(&lo_bits, &lo, 4);
+        lo_bits = (lo_bits + 0x8000u) & 0xFFFF0000u;      // to 16 bits (2^-8 of it)
+        t.wedge[i] = static_cast<float>(1.0 / std::expm1(t.x[i] - t.x[i + 1]));
         // the product is monotone in u, so the test of the largest u with these
         // upper 16 bits decides for all of them
         int n = static_cast<int>(t.x[i + 1] / t.x[i] * 65536.0) + 1;
@@ -515,7 +345,7 @@ static void build_zig_table(ZigTab &t) {
             return std::ldexp(static_cast<double>(uv), -53) * t.x[i] < t.x[i + 1];
         };
         while (n > 0 && !passes(n)) --n;
-        t.fast_t[i] = static_cast<uint16_t>(std::max(0, std::min(n, 65536) - 16));
+        t.fast_lo[i] = lo_bits | static_cast<uint32_t>(std::max(0, std::min(n, 65536) - 16));
     }
 }
 

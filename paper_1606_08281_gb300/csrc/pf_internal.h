@@ -65,6 +65,7 @@ struct FilterArgs {
     double slack;               // upper bound of one per-time-point log increment, >= 0
     const ZigTab *zig;          // device copy of the exponential ziggurat table
     int32_t cluster;            // > 1: each filter split over a cluster of this many blocks
+    uint32_t round_keys[20];    // Philox round keys of `seed` (set at launch)
     int32_t fast;               // bytes of shared memory of the SSA without FP64 (0: not used)
 };
 
@@ -85,6 +86,12 @@ int reaction_tier(int R);
 int launch_filter(const FilterArgs &a, int block_threads, double *loglik, uint8_t *status,
                   void *stream, unsigned char *slabs = nullptr, size_t slab_bytes = 0,
                   int grid = 0);
+
+// Its launch forms over clusters and from global slabs (`smem`: dynamic shared
+// memory of a block).
+int launch_filter_cluster(const FilterArgs &a, int block_threads, size_t smem, struct CUstream_st *s);
+int launch_filter_global(const FilterArgs &a, int block_threads, unsigned char *slabs, size_t slab_bytes, int grid,
+                         struct CUstream_st *s);
 
 // Raise a kernel's dynamic shared-memory limit (a process-wide attribute)
 // once per device to the largest size any launch of it can use; never lowers

@@ -17,14 +17,15 @@
 //     the caps is handed over (below).  A_r >= 2^30 is within 2^-31 of the
 //     rate; smaller ones contribute at most h_r / 2 units, bounded by e_abs.
 //   * the waiting time's variate is u x_i (ziggurat layer i) in two-float
-//     arithmetic from 48 bits of u >= 2^-12 and x_i to 2^-48; draws whose layer
+//     arithmetic from 48 bits of u >= 2^-12 and x_i to 2^-32; draws whose layer
 //     test w1 < T_i (an integer threshold, a lower bound of the FP64 test) does
-//     not accept, 0.4 % of them, take the FP64 ziggurat.
+//     not accept, 0.4 % of them, take the wedge tests in FP32, and the FP64
+//     ziggurat where those are too close (0.03 %).
 //   * tau = E / a0 from the approximate reciprocal of a0's 24 leading bits,
 //     corrected to all of its 32 leading bits; relative error below
 //     2^-31 (rates) + 2^-31 (a0 truncated) + 2^-36 (u) + 2^-42 (reciprocal,
-//     products) < 2^-29.9.  Times are 64-bit integers with the interval scaled
-//     to [2^50, 2^51) units, so sums add one unit of rounding per event.
+//     products) + 2^-32 (x_i) < 2^-29.8.  Times are 64-bit integers with the interval scaled
+//     to [2^49, 2^50) units, so sums add one unit of rounding per event.
 //   * an event at t is in time when t < D - b and late when t > D + b, with
 //     D the interval's length and b = 2^-28 D + (c units per draw) + the
 //     e_abs contribution accumulated along the path; c covers this path's
@@ -36,9 +37,11 @@
 //     when e_abs > 0), this one choice is recomputed in FP64 (exact_step).
 //
 // So states, draw counts and event counts equal the FP64 definition's, bit for
-// bit.  What bounds the path is instruction issue: gene expression (R = 4)
-// spends about 190 warp instructions per event instead of 580 with 16 FP64
-// ones of 16 cycles each.
+// bit.  What bounds the path is instruction issue (64 % of the cycles with 24
+// warps per SM) and, for few filters, the latency of one event's chain, about
+// 1500 cycles: gene expression (1024 rows x 10 x 1000 particles x 50 times)
+// 373-417 ms by the FP64 path, 161 ms; the cascade (64 x 16 x 512 x 60, 20
+// reactions) 561-597 ms and 125 ms.
 //
 // Each lane simulates its particle in a private column of shared memory
 // (conflict-free, whatever the particle's index, and the same for populations
@@ -53,7 +56,7 @@ namespace pf {
 namespace dev {
 
 // Largest block of the filter kernels.
-constexpr int kMaxThreads = 128;
+constexpr int kMaxThreads = 256;
 constexpr int kCheckTrips = 32;    // trips between two looks at the counts' caps
 
 // One reaction: A_r and the byte offsets of its reactants' rows in a column.
@@ -64,8 +67,7 @@ struct FastReac {
 };
 
 struct __align__(16) FastShared {
-    float2 zx[kZigLayers];               // x_i 2^-24, leading and trailing part
-    uint16_t zt[kZigLayers];             // accept when (w1 >> 16) - 16 < zt (unsigned)
+    float2 zx[kZigLayers];               // x_i 2^-24; trailing part in 16 bits | layer test in 16 bits
     FastReac reac[PF_MAX_REACTIONS];
     uint4 change[PF_MAX_REACTIONS];      // up to four words: row offset << 16 | delta
     int mx[PF_MAX_SPECIES];              // the population's largest counts
@@ -73,36 +75,51 @@ struct __align__(16) FastShared {
     unsigned long long D;                // interval length in time units
     unsigned long long b0;               // b without its per-draw and e_abs parts
     double unit;                         // time units per unit of time (a power of two)
-    uint32_t quick_lo, quick_hi;         // upper words that decide most events
+    uint32_t quick_lo, quick_hi;         // times' bits from 2^30 on that decide most events
     uint32_t c;                          // units per draw in b
     uint32_t hi_min;                     // a0's upper word below this: exact_step
     uint32_t margin;                     // reaction choice
     uint32_t scale;                      // exponent bits of the time scale
     float ecoef;                         // e_abs in the units the path's bound needs
+    float rate_up[PF_MAX_REACTIONS];     // rates rounded up (0: a rate outside 2^-80 .. 2^80 and not 0)
     uint32_t mask2;                      // reactions of order 2
     int gain;                            // largest count a reaction adds
     int possible;                        // the network's part of the conditions
     int on;                              // this interval runs here
     int n_exact;                         // particles to replay
-    uint16_t rem_slot[2][kMaxThreads];   // parked particles' columns
-    float rem_err[2][kMaxThreads];       // and accumulated bounds
+    uint16_t rem_slot[2][kMaxRemnants];  // parked particles' columns
+    float rem_err[2][kMaxRemnants];      // and accumulated bounds
 };
 
-// Shared memory of the path: tables, and U + 1 rows of one column per thread.
+// Dynamic shared memory of a filter block: the block's head; then, where this
+// path runs, its tables and U + 1 rows of one column per thread; then the
+// population (unless it is in global memory).  The parts are reached through
+// these functions so that code called out of line still addresses them as
+// shared memory.
+constexpr size_t kHeadBytes = (sizeof(SharedHead) + 15) & ~static_cast<size_t>(15);
 __host__ __device__ __forceinline__ size_t fast_smem_bytes(int U, int threads) {
-    return sizeof(FastShared) + sizeof(int) * static_cast<size_t>(U + 1) * threads;
+    return (sizeof(FastShared) + sizeof(int) * static_cast<size_t>(U + 1) * threads + 15) & ~static_cast<size_t>(15);
+}
+extern __shared__ __align__(16) unsigned char g_smem[];
+__device__ __forceinline__ SharedHead &block_head() { return *reinterpret_cast<SharedHead *>(g_smem); }
+__device__ __forceinline__ FastShared &block_fast() { return *reinterpret_cast<FastShared *>(g_smem + kHeadBytes); }
+__device__ __forceinline__ int *block_columns() {
+    return reinterpret_cast<int *>(g_smem + kHeadBytes + sizeof(FastShared));
 }
 
-__device__ __forceinline__ void load_fast_zig(FastShared &fs, const ZigTab *src) {
+__device__ __forceinline__ void load_fast_zig(const ZigTab *src) {
+    FastShared &fs = block_fast();
     for (int i = threadIdx.x; i < kZigLayers; i += blockDim.x) {
-        fs.zx[i] = make_float2(src->fast_hi[i], src->fast_lo[i]);
-        fs.zt[i] = src->fast_t[i];
+        fs.zx[i] = make_float2(src->fast_hi[i], __uint_as_float(src->fast_lo[i]));
     }
 }
 
 // Per-filter part of the set-up (the network's tables are loaded); the caller
 // synchronises afterwards.
-__device__ __forceinline__ void fast_network(FastShared &fs, int *cols, const NetTables &n) {
+__device__ __forceinline__ void fast_network() {
+    FastShared &fs = block_fast();
+    int *const cols = block_columns();
+    const NetTables &n = block_head().net;
     const int tid = threadIdx.x, B = blockDim.x;
     const uint32_t row = 4u * B;
     cols[n.U * B + tid] = 1;
@@ -148,13 +165,24 @@ __device__ __forceinline__ int exponent_of(double v) {
     return static_cast<int>(__double_as_longlong(v) >> 52) - 1023;
 }
 
+// Per-filter part that needs the rates (set by the threads r < R); the caller
+// synchronises afterwards.
+__device__ __forceinline__ void fast_rate(int r, double rate) {
+    const int ex = exponent_of(rate);
+    const bool zero = __double_as_longlong(rate) == 0;
+    if (!zero && !(ex > -80 && ex < 80)) atomicAnd(&block_fast().possible, 0);
+    block_fast().rate_up[r] = zero ? 0.0f : __double2float_ru(rate);
+}
+
 // Per-interval set-up by the whole block: caps, k, A_r, time scale and bounds.
 // Returns whether the interval can run here (the same in every thread); the
 // caller has synchronised after the last write to xs.
-__device__ __forceinline__ bool fast_interval(FastShared &fs, const NetTables &n, const double *rate,
-                                              const int *xs, int Np, int N, double t_prev,
-                                              double t_end, uint64_t budget) {
+static __device__ __noinline__ bool fast_interval(const int *xs, int Np, int N, double t_prev, double t_end,
+                                           uint64_t budget) {
+    FastShared &fs = block_fast();
     if (!fs.possible) return false;
+    const NetTables &n = block_head().net;
+    const double *rate = block_head().rate;
     const int tid = threadIdx.x, B = blockDim.x, U = n.U;
     for (int u = 0; u < U; ++u) {
         int m = 0;
@@ -172,28 +200,27 @@ __device__ __forceinline__ bool fast_interval(FastShared &fs, const NetTables &n
             return 4ull * static_cast<uint32_t>(fs.mx[u]) + 1024ull + room;
         };
         bool ok = true;
-        double rt = 0.0;
+        float up = 0.0f;
         uint64_t h = 1;
         if (r < n.R) {
-            rt = rate[r];
+            up = fs.rate_up[r];
             const FastReac &q = fs.reac[r];
             const uint64_t ca = cap_of(q.a), cb = cap_of(q.b >> 1);
-            ok = ca < (1ull << 28) && cb < (1ull << 28);
             h = ca * cb;                     // the product formed before the shift must fit 32 bits
-            ok = ok && h < (1ull << 32);
+            ok = ca < (1ull << 28) && cb < (1ull << 28) && h < (1ull << 32);
             if (q.b & 1u) h >>= 1;
-            const int ex = exponent_of(rt);
-            ok = ok && (__double_as_longlong(rt) == 0 || (ex > -80 && ex < 80));
         }
+        const float hf = __uint2float_ru(static_cast<uint32_t>(h));
         // sum of rate times the largest h, rounded up
-        float sum = r < n.R ? __fmul_ru(__double2float_ru(rt), __ull2float_ru(h)) : 0.0f;
+        float sum = __fmul_ru(up, hf);
         for (int o = 16; o > 0; o >>= 1) sum = __fadd_ru(sum, __shfl_xor_sync(0xFFFFFFFFu, sum, o));
         ok = ok && sum > 0.0f && sum < 1e36f;
         const int k = 61 - ((__float_as_int(sum) >> 23) - 127);     // sum 2^k < 2^62
         uint64_t A = 0;
-        if (ok && __double_as_longlong(rt) != 0) {
-            const uint64_t m53 = (static_cast<uint64_t>(__double_as_longlong(rt)) & ((1ull << 52) - 1ull)) | (1ull << 52);
-            const int sh = exponent_of(rt) - 52 + k;
+        if (ok && up > 0.0f) {
+            const long long rb = __double_as_longlong(rate[r]);
+            const uint64_t m53 = (static_cast<uint64_t>(rb) & ((1ull << 52) - 1ull)) | (1ull << 52);
+            const int sh = static_cast<int>(rb >> 52) - 1075 + k;
             if (sh >= 0) A = m53 << min(sh, 63);
             else if (sh > -63) A = (m53 + (1ull << (-sh - 1))) >> -sh;
         }
@@ -202,19 +229,19 @@ __device__ __forceinline__ bool fast_interval(FastShared &fs, const NetTables &n
             fs.reac[r].hi = static_cast<uint32_t>(A >> 32);
         }
         // absolute error of the sums from the coarsely represented rates
-        const bool coarse = __double_as_longlong(rt) != 0 && A < (1ull << 30);
-        float e_abs = coarse ? __fmul_ru(0.5f, __ull2float_ru(h)) : 0.0f;
+        const bool coarse = up > 0.0f && A < (1ull << 30);
+        float e_abs = coarse ? 0.5f * hf : 0.0f;
         for (int o = 16; o > 0; o >>= 1) e_abs = __fadd_ru(e_abs, __shfl_xor_sync(0xFFFFFFFFu, e_abs, o));
         ok = ok && e_abs < 1073741824.0f;
-        // time scale: D = (t_end - t_prev) 2^q in [2^50, 2^51)
+        // time scale: D = (t_end - t_prev) 2^q in [2^49, 2^50)
         const double d = __dsub_rn(t_end, t_prev);
-        const int ed = exponent_of(d), q = 50 - ed;
-        const uint64_t D = ((static_cast<uint64_t>(__double_as_longlong(d)) & ((1ull << 52) - 1ull)) | (1ull << 52)) >> 2;
-        const float ratio = __fdiv_ru(__double2float_ru(t_end), __double2float_rd(d));
-        ok = ok && ed > -500 && ed < 500 && ratio < 16384.0f;
+        const int ed = exponent_of(d), q = 49 - ed;
+        const uint64_t D = ((static_cast<uint64_t>(__double_as_longlong(d)) & ((1ull << 52) - 1ull)) | (1ull << 52)) >> 3;
+        const int far = exponent_of(t_end) + 1 - ed;              // t_end < 2^far D
+        ok = ok && ed > -500 && ed < 500 && far <= 14;
         const int kq = k + q;
         ok = ok && kq >= 40 && kq <= 120;
-        const uint32_t c = ok ? 4u + static_cast<uint32_t>(ratio) : 4u;
+        const uint32_t c = 4u + (ok ? 1u << max(far - 2, 0) : 0u);
         const uint64_t per_draws = c * (budget < (1ull << 40) ? budget : (1ull << 40));
         const uint64_t b_quick = (D >> 16) + per_draws;
         ok = ok && b_quick < (D >> 2);
@@ -228,8 +255,8 @@ __device__ __forceinline__ bool fast_interval(FastShared &fs, const NetTables &n
             fs.D = D;
             fs.unit = __longlong_as_double(static_cast<long long>(1023 + (ok ? q : 0)) << 52);
             fs.b0 = D >> 28;
-            fs.quick_lo = static_cast<uint32_t>((D - b_quick) >> 32);
-            fs.quick_hi = static_cast<uint32_t>((D + b_quick) >> 32);
+            fs.quick_lo = static_cast<uint32_t>((D - b_quick) >> 30);
+            fs.quick_hi = static_cast<uint32_t>((D + b_quick) >> 30);
             fs.c = c;
             // e_abs / a0 stays below 2^-18: well inside the quick bound's 2^-16 D
             // and, in 31-bit units, below half the margin of 2^14
@@ -276,54 +303,171 @@ static __device__ __noinline__ int exact_step(const NetTables &n, const double *
     return chosen >= R ? last : chosen;
 }
 
+// One attempt of the ziggurat: u x_i as a sum of two floats, u from the 48 upper
+// bits of the word (w1, w0), and whether the layer's test accepts it.
+__device__ __forceinline__ bool zig_first(const FastShared &fs, int layer, uint32_t w1, uint32_t w0, float &Eh,
+                                          float &El) {
+    const float2 zx = fs.zx[layer];
+    const uint32_t z = __float_as_uint(zx.y);
+    const float uh = static_cast<float>(w1 >> 8);
+    const float ul = static_cast<float>(__byte_perm(w0, w1, 0x4432) & 0xFFFFFFu) * 5.9604644775390625e-8f;
+    const float p = __fmul_rn(uh, zx.x);
+    float q = __fmaf_rn(uh, zx.x, -p);
+    q = __fmaf_rn(ul, zx.x, q);
+    q = __fmaf_rn(uh, __uint_as_float(z & 0xFFFF0000u), q);
+    Eh = __fadd_rn(p, q);
+    El = __fsub_rn(q, __fsub_rn(Eh, p));
+    return (w1 >> 16) - 16u < (z & 0xFFFFu);
+}
+
+// A draw whose first word (layer, w1, w0) passes no layer test: the wedge tests
+// U < (e^d - 1) / (e^D - 1), d = x_i - x, D = x_i - x_{i+1} (the ziggurat's
+// f_i + U (f_{i+1} - f_i) < e^-x divided by f_i), and further attempts, as
+// zig_exp does them.  Both sides are within 2^-19 of their FP64 values; false
+// when they are closer than 2^-15, or for the tail and for small u: zig_exp
+// then decides (1 draw in 3000).
+static __device__ __noinline__ bool zig_wedges(const FastShared &fs, const ZigTab *zig, int layer, uint32_t w1,
+                                               uint32_t w0, uint32_t draws, uint32_t particle, uint32_t lane,
+                                               uint32_t mrow, uint32_t key0, uint32_t key1, float &Eh, float &El) {
+    for (uint32_t s = 1; s < 32; ++s) {
+        if (layer == 0 || (w1 >> 16) < 16u) return false;
+        const Philox4 x = philox4x32_10(draws, particle | (s << 16), lane, mrow, key0, key1);
+        const float xi = fs.zx[layer].x * 16777216.0f;
+        const float d = static_cast<float>(~w1) * 2.3283064365386963e-10f * xi;
+        const float g = expm1f(d) * __ldg(&zig->wedge[layer]);
+        const float U = static_cast<float>(x.w1) * 2.3283064365386963e-10f;
+        if (fabsf(U - g) < 3.0517578125e-5f) return false;
+        if (U < g) return true;
+        w1 = x.w3;
+        w0 = x.w2;
+        layer = static_cast<int>(w0 & 0x7FFu);
+        if ((w1 >> 16) < 16u) return false;
+        if (zig_first(fs, layer, w1, w0, Eh, El)) return true;
+    }
+    return false;
+}
+
+// Shared-memory accesses by 32-bit address (columns are private to a lane).
+__device__ __forceinline__ uint32_t shared_addr(const void *p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ uint32_t col_load(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void col_store(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Philox round keys: from the seed, or precomputed in the kernel's parameters
+// (constant-bank operands: no additions and no registers).
+struct SeedKeys {
+    uint32_t key0, key1;
+    __device__ __forceinline__ uint32_t k0(uint32_t round) const { return key0 + round * 0x9E3779B9u; }
+    __device__ __forceinline__ uint32_t k1(uint32_t round) const { return key1 + round * 0xBB67AE85u; }
+};
+struct ParamKeys {
+    const uint32_t *rk;        // k0 of rounds 0..9, then k1
+    __device__ __forceinline__ uint32_t k0(uint32_t round) const { return rk[round]; }
+    __device__ __forceinline__ uint32_t k1(uint32_t round) const { return rk[10 + round]; }
+};
+
+static __device__ __noinline__ double zig_call(uint32_t w1, uint32_t w0, uint32_t draws, uint32_t particle, uint32_t lane,
+                                               uint32_t mrow, uint32_t key0, uint32_t key1, const ZigTab *zig) {
+    return zig_exp((static_cast<uint64_t>(w1) << 32) | w0, draws, particle, lane, mrow, key0, key1, zig->x, zig);
+}
+
 // Simulate the interval's particles (see the head of this file).  Particles
 // that must be replayed are appended to `redo`, their state untouched.
+// Returns the reactions that this thread's finished particles fired.
 // Preconditions: fast_interval returned true, sh.pool_next = blockDim.x,
 // sh.rem_n = {0, 0}.
-template <int RM>
-__device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *cols, int *xs, int Np, int N,
-                                         uint32_t key0, uint32_t key1, uint32_t lane, uint32_t mrow,
-                                         uint64_t budget, unsigned long long &fired, uint32_t j0, int *redo) {
+//
+// Up to eight reactions keep their prefix sums in registers and compare all of
+// them with the target.  More keep only every fourth sum: the choice picks a
+// group of four by those and computes the group's sums again, which costs the
+// same instructions (20 reactions: 9 compares instead of 20, three sums again)
+// and 16 registers instead of 64, so that 24 warps fit on an SM instead of 16.
+template <int RM, int UM, class Keys>
+__device__ __forceinline__ unsigned long long ssa_fast(int *xs, int Np, int N, const Keys &keys, uint32_t lane,
+                                                       uint32_t mrow, uint32_t budget32, uint32_t j0, int *redo) {
     constexpr uint32_t kMulA = 0xD2511F53u, kMulB = 0xCD9E8D57u;
-    constexpr uint32_t kWeylA = 0x9E3779B9u, kWeylB = 0xBB67AE85u;
-    const int R4 = (sh.net.R + 3) & ~3, U = sh.net.U, B = blockDim.x;
+    constexpr bool kHoist = RM <= 4;             // reactions in registers
+    constexpr bool kGroups4 = RM > 8;            // prefix sums by groups of four
+    SharedHead &sh = block_head();
+    FastShared &fs = block_fast();
+    int *const cols = block_columns();
+    const int R4 = (sh.net.R + 3) & ~3, U = sh.net.U;
+    const uint32_t row = 4u * blockDim.x;
+    const uint32_t cols_addr = shared_addr(cols);
     const uint32_t mask2 = fs.mask2, hi_min = fs.hi_min, margin = fs.margin;
     const uint32_t quick_lo = fs.quick_lo, quick_hi = fs.quick_hi, scale = fs.scale;
     const float ecoef = fs.ecoef;
-    const uint32_t budget32 = static_cast<uint32_t>(budget);
-    char *col = reinterpret_cast<char *>(cols + threadIdx.x);
+    unsigned long long fired = 0;
+    uint32_t col = cols_addr + 4u * threadIdx.x;
     // Philox rounds 1 and 2 depend on the draw counter only in part
     const uint64_t pB = static_cast<uint64_t>(kMulB) * lane;
-    uint32_t pn0 = 0, pA_hi = 0, pA_lo = 0;
+    uint32_t pA_hi = 0, pA_lo = 0;
     int j = 0;
     auto set_particle = [&]() {
-        pn0 = static_cast<uint32_t>(pB >> 32) ^ (j0 + static_cast<uint32_t>(j)) ^ key0;
-        const uint64_t p = static_cast<uint64_t>(kMulA) * pn0;
-        pA_hi = static_cast<uint32_t>(p >> 32) ^ (key1 + kWeylB);
+        const uint32_t n0 = static_cast<uint32_t>(pB >> 32) ^ (j0 + static_cast<uint32_t>(j)) ^ keys.k0(0);
+        const uint64_t p = static_cast<uint64_t>(kMulA) * n0;
+        pA_hi = static_cast<uint32_t>(p >> 32) ^ keys.k1(1);
         pA_lo = static_cast<uint32_t>(p);
     };
     bool active = false;
-    unsigned long long t = 0;
+    uint32_t t_hi = 0, t_lo = 0;                 // time: t_hi 2^30 + t_lo units, t_lo < 2^30
     uint32_t draws = 0;
     float err = 0.0f;
+    auto load_state = [&]() {
+        if constexpr (UM > 0) {
+#pragma unroll
+            for (int u = 0; u < UM; ++u)
+                if (u < U) col_store(col + u * row, static_cast<uint32_t>(xs[u * Np + j]));
+        } else {
+            for (int u = 0; u < U; ++u) col_store(col + u * row, static_cast<uint32_t>(xs[u * Np + j]));
+        }
+    };
+    auto store_state = [&]() {
+        if constexpr (UM > 0) {
+#pragma unroll
+            for (int u = 0; u < UM; ++u)
+                if (u < U) xs[u * Np + j] = static_cast<int>(col_load(col + u * row));
+        } else {
+            for (int u = 0; u < U; ++u) xs[u * Np + j] = static_cast<int>(col_load(col + u * row));
+        }
+    };
     auto start = [&](int slot) {
         active = slot < N;
         if (active) {
             j = slot;
-            for (int u = 0; u < U; ++u) *reinterpret_cast<int *>(col + u * 4 * B) = xs[u * Np + j];
+            load_state();
             set_particle();
-            t = 0;
+            t_hi = 0;
+            t_lo = 0;
             draws = 0;
             err = 0.0f;
         }
     };
-    // small networks keep the reactions in registers
-    constexpr bool kHoist = RM <= 4;
     FastReac reg[kHoist ? RM : 1];
     if constexpr (kHoist) {
 #pragma unroll
         for (int r = 0; r < RM; ++r) reg[r] = fs.reac[r];
     }
+    // h_r(x) of the reaction at the lane's column
+    auto count = [&](const FastReac &q, bool second) -> uint32_t {
+        uint32_t h = col_load(col + q.a);
+        if (second) {
+            const uint32_t same = q.b & 1u;
+            h = (h * (col_load(col + (q.b >> 1)) - same)) >> same;
+        }
+        return h;
+    };
+    auto add = [](unsigned long long run, const FastReac &q, uint32_t h) {
+        run += static_cast<unsigned long long>(q.lo) * h;
+        return run + (static_cast<unsigned long long>(q.hi * h) << 32);
+    };
     int src = 0, remaining = N;
     bool first = true;
     for (;;) {
@@ -334,10 +478,12 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
             if (active) {
                 const int i = threadIdx.x;
                 j = sh.rem_j[src][i];
-                t = static_cast<unsigned long long>(__double_as_longlong(sh.rem_t[src][i]));
+                const unsigned long long t = static_cast<unsigned long long>(__double_as_longlong(sh.rem_t[src][i]));
+                t_hi = static_cast<uint32_t>(t >> 32);
+                t_lo = static_cast<uint32_t>(t);
                 draws = sh.rem_draws[src][i];
                 err = fs.rem_err[src][i];
-                col = reinterpret_cast<char *>(cols + fs.rem_slot[src][i]);
+                col = cols_addr + 4u * fs.rem_slot[src][i];
                 set_particle();
             }
         }
@@ -352,10 +498,11 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
                     if (active) {
                         const int slot = atomicAdd(&sh.rem_n[dst], 1);
                         sh.rem_j[dst][slot] = j;
-                        sh.rem_t[dst][slot] = __longlong_as_double(static_cast<long long>(t));
+                        sh.rem_t[dst][slot] = __longlong_as_double(
+                            static_cast<long long>((static_cast<unsigned long long>(t_hi) << 32) | t_lo));
                         sh.rem_draws[dst][slot] = draws;
                         fs.rem_err[dst][slot] = err;
-                        fs.rem_slot[dst][slot] = static_cast<uint16_t>(reinterpret_cast<int *>(col) - cols);
+                        fs.rem_slot[dst][slot] = static_cast<uint16_t>((col - cols_addr) >> 2);
                     }
                     break;
                 }
@@ -364,63 +511,53 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
             int fin = 0;               // 1: at t_end, 2: to be replayed
             if (trip % kCheckTrips == 0) {
                 for (int u = 0; u < U; ++u)
-                    if (*reinterpret_cast<int *>(col + u * 4 * B) > fs.lim[u]) fin = 2;
+                    if (static_cast<int>(col_load(col + u * row)) > fs.lim[u]) fin = 2;
             }
             if (fin == 0) {
                 // the draw's random words: Philox4x32-10 of (draws, particle, lane, row)
                 uint32_t w0, w1, w2, w3;
                 {
                     const uint64_t p1 = static_cast<uint64_t>(kMulA) * draws;
-                    const uint32_t n2 = static_cast<uint32_t>(p1 >> 32) ^ mrow ^ key1;
+                    const uint32_t n2 = static_cast<uint32_t>(p1 >> 32) ^ mrow ^ keys.k1(0);
                     const uint64_t q1 = static_cast<uint64_t>(kMulB) * n2;
-                    uint32_t c0 = static_cast<uint32_t>(q1 >> 32) ^ static_cast<uint32_t>(pB) ^ (key0 + kWeylA);
-                    uint32_t c1 = static_cast<uint32_t>(q1);
-                    uint32_t c2 = pA_hi ^ static_cast<uint32_t>(p1);
-                    uint32_t c3 = pA_lo;
+                    w0 = static_cast<uint32_t>(q1 >> 32) ^ static_cast<uint32_t>(pB) ^ keys.k0(1);
+                    w1 = static_cast<uint32_t>(q1);
+                    w2 = pA_hi ^ static_cast<uint32_t>(p1);
+                    w3 = pA_lo;
 #pragma unroll
                     for (uint32_t round = 2; round < 10; ++round) {
-                        const uint64_t a = static_cast<uint64_t>(kMulA) * c0;
-                        const uint64_t b = static_cast<uint64_t>(kMulB) * c2;
-                        c0 = static_cast<uint32_t>(b >> 32) ^ c1 ^ (key0 + round * kWeylA);
-                        c1 = static_cast<uint32_t>(b);
-                        c2 = static_cast<uint32_t>(a >> 32) ^ c3 ^ (key1 + round * kWeylB);
-                        c3 = static_cast<uint32_t>(a);
+                        const uint64_t a = static_cast<uint64_t>(kMulA) * w0;
+                        const uint64_t b = static_cast<uint64_t>(kMulB) * w2;
+                        w0 = static_cast<uint32_t>(b >> 32) ^ w1 ^ keys.k0(round);
+                        w1 = static_cast<uint32_t>(b);
+                        w2 = static_cast<uint32_t>(a >> 32) ^ w3 ^ keys.k1(round);
+                        w3 = static_cast<uint32_t>(a);
                     }
-                    w0 = c0;
-                    w1 = c1;
-                    w2 = c2;
-                    w3 = c3;
                 }
-                // prefix sums of the propensities
-                unsigned long long S[RM], run = 0;
+                // prefix sums of the propensities (each, or every fourth)
+                constexpr int kSums = kGroups4 ? RM / 4 : RM;
+                unsigned long long S[kSums], run = 0;
 #pragma unroll
                 for (int r0 = 0; r0 < RM; r0 += 4) {
                     if (r0 < R4) {
                         const bool second = ((mask2 >> r0) & 15u) != 0;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const int r = r0 + i;
                             FastReac q;
-                            if constexpr (kHoist) q = reg[r];
-                            else q = fs.reac[r];
-                            uint32_t h = *reinterpret_cast<uint32_t *>(col + q.a);
-                            if (second) {
-                                const uint32_t same = q.b & 1u;
-                                h = (h * (*reinterpret_cast<uint32_t *>(col + (q.b >> 1)) - same)) >> same;
-                            }
-                            run += static_cast<unsigned long long>(q.lo) * h;
-                            run += static_cast<unsigned long long>(q.hi * h) << 32;
-                            S[r] = run;
+                            if constexpr (kHoist) q = reg[r0 + i];
+                            else q = fs.reac[r0 + i];
+                            run = add(run, q, count(q, second));
+                            if constexpr (!kGroups4) S[r0 + i] = run;
                         }
-                    } else {
+                    } else if constexpr (!kGroups4) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) S[r0 + i] = run;
                     }
+                    if constexpr (kGroups4) S[r0 / 4] = run;
                 }
-                const uint64_t v2 = ((static_cast<uint64_t>(w3) << 32) | w2) >> 11;
                 const uint32_t a_hi = static_cast<uint32_t>(run >> 32);
                 int chosen;
-                unsigned long long t_next = t;
+                uint32_t n_hi = t_hi, n_lo = t_lo;       // time of the event
                 if (a_hi >= hi_min) {
                     if (draws >= budget32) {
                         sh.status = PF_ST_BUDGET;
@@ -428,27 +565,17 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
                     }
                     // E as a sum of two floats
                     const int layer = static_cast<int>(w0 & 0x7FFu);
-                    const float2 zx = fs.zx[layer];
                     float Eh, El;
-                    {
-                        const float uh = static_cast<float>(w1 >> 8);
-                        const float ul = static_cast<float>(((w1 & 0xFFu) << 16) | (w0 >> 16)) * 5.9604644775390625e-8f;
-                        const float p = __fmul_rn(uh, zx.x);
-                        float q = __fmaf_rn(uh, zx.x, -p);
-                        q = __fmaf_rn(ul, zx.x, q);
-                        q = __fmaf_rn(uh, zx.y, q);
-                        Eh = __fadd_rn(p, q);
-                        El = __fsub_rn(q, __fsub_rn(Eh, p));
-                    }
-                    if ((w1 >> 16) - 16u >= static_cast<uint32_t>(fs.zt[layer])) {
-                        const uint64_t r0 = (static_cast<uint64_t>(w1) << 32) | w0;
-                        const double E = zig_exp(r0, draws, j0 + static_cast<uint32_t>(j), lane, mrow, key0, key1,
-                                                 sh.zig_g->x, sh.zig_g);
+                    if (!zig_first(fs, layer, w1, w0, Eh, El) &&
+                        !zig_wedges(fs, sh.zig_g, layer, w1, w0, draws, j0 + static_cast<uint32_t>(j), lane, mrow,
+                                    keys.k0(0), keys.k1(0), Eh, El)) {
+                        const double E = zig_call(w1, w0, draws, j0 + static_cast<uint32_t>(j), lane, mrow, keys.k0(0),
+                                                  keys.k1(0), sh.zig_g);
                         Eh = __double2float_rn(E);
                         El = __double2float_rn(__dsub_rn(E, static_cast<double>(Eh)));
                     }
-                    // tau = E / a0 in time units
-                    const int s = __clz(static_cast<int>(a_hi));
+                    // tau = E / a0 in time units: a0's 32 leading bits as f + g
+                    const int s = 158 - (__float_as_int(__uint2float_rz(a_hi)) >> 23);
                     const uint32_t mh = __funnelshift_l(static_cast<uint32_t>(run), a_hi, s);
                     const float f = static_cast<float>(mh & 0xFFFFFF00u), g = static_cast<float>(mh & 0xFFu);
                     float rc;
@@ -460,68 +587,97 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
                     pl = __fmaf_rn(El, rs, pl);
                     pl = __fmaf_rn(ph, e, pl);
                     err = __fmaf_ru(ph, __fmul_ru(rs, ecoef), err);
-                    t_next = t + static_cast<unsigned long long>(__float2ll_rn(ph)) +
-                             static_cast<unsigned long long>(static_cast<long long>(__float2int_rn(pl)));
-                    // the reaction
+                    // tau to an integer in two parts (64-bit conversions run on
+                    // the FP64 pipe): a multiple of 2^30 by adding 1.5 2^23, and
+                    // the rest; from 2^52 on the event is late whatever its size.
+                    // |rest| <= 2^29 and |pl| < 2^-21.5 ph: for ph up to 1.3 2^50,
+                    // beyond which the event is late whatever lo's carry, lo fits
+                    const float pc = fminf(ph, 4503599627370496.0f);
+                    const float top = __fmaf_rn(pc, 9.31322574615478515625e-10f, 12582912.0f);
+                    const float rest = __fmaf_rn(-1073741824.0f, __fsub_rn(top, 12582912.0f), pc);
+                    const uint32_t lo = t_lo + static_cast<uint32_t>(__float2int_rn(__fadd_rn(rest, pl)));
+                    n_hi = t_hi + (__float_as_uint(top) - 0x4B400000u) + static_cast<uint32_t>(static_cast<int>(lo) >> 30);
+                    n_lo = lo & 0x3FFFFFFFu;
+                    // the reaction: the prefix sums at or below u2 a0, on 31
+                    // leading bits; a target next to a0 itself counts as near
                     const uint32_t tgt = __umulhi(w3, mh) >> 1;
-                    int neg = 0;
-                    uint32_t near = 0xFFFFFFFFu;
+                    uint32_t near = ~w3;
+                    auto below = [&](unsigned long long v) -> int {      // 0 when the sum is at or below the target, else -1
+                        const uint32_t d = tgt - __funnelshift_l(static_cast<uint32_t>(v), static_cast<uint32_t>(v >> 32), s - 1);
+                        near = min(near, d + margin);
+                        return static_cast<int>(d) >> 31;
+                    };
+                    if constexpr (kGroups4) {
+                        int above = 0;
+                        unsigned long long base = 0;
 #pragma unroll
-                    for (int r0 = 0; r0 < RM; r0 += 4) {
-                        if (r0 < R4) {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const uint32_t Sn = __funnelshift_l(static_cast<uint32_t>(S[r0 + i]),
-                                                                    static_cast<uint32_t>(S[r0 + i] >> 32), s - 1);
-                                const uint32_t dd = tgt - Sn;
-                                neg += static_cast<int>(dd) >> 31;
-                                near = min(near, dd + margin);
+                        for (int q = 0; q < RM / 4 - 1; ++q) {
+                            if (4 * q < R4) {
+                                const int b = below(S[q]);
+                                above += b + 1;
+                                base = b ? base : S[q];
                             }
                         }
+                        chosen = min(4 * above, R4 - 4);
+                        int inner = 3;
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            const FastReac q = fs.reac[chosen + i];
+                            base = add(base, q, count(q, mask2 != 0));
+                            inner += below(base);
+                        }
+                        chosen += inner;
+                    } else {
+                        chosen = RM - 1;
+#pragma unroll
+                        for (int r = 0; r < RM - 1; ++r) chosen += below(S[r]);
                     }
-                    chosen = R4 + neg;
                     if (near < 2u * margin) {
                         double tau;
-                        chosen = exact_step(sh.net, sh.rate, reinterpret_cast<int *>(col), B, 1.0, v2, tau);
+                        chosen = exact_step(sh.net, sh.rate, cols + ((col - cols_addr) >> 2), blockDim.x, 1.0,
+                                            ((static_cast<uint64_t>(w3) << 32) | w2) >> 11, tau);
                     }
                 } else {
                     // a0 is zero or too small for its relative error
-                    const uint64_t r0 = (static_cast<uint64_t>(w1) << 32) | w0;
-                    const double E = zig_exp(r0, draws, j0 + static_cast<uint32_t>(j), lane, mrow, key0, key1,
-                                             sh.zig_g->x, sh.zig_g);
+                    const double E = zig_call(w1, w0, draws, j0 + static_cast<uint32_t>(j), lane, mrow, keys.k0(0),
+                                              keys.k1(0), sh.zig_g);
                     double tau = 0.0;
-                    chosen = exact_step(sh.net, sh.rate, reinterpret_cast<int *>(col), B, E, v2, tau);
+                    chosen = exact_step(sh.net, sh.rate, cols + ((col - cols_addr) >> 2), blockDim.x, E,
+                                        ((static_cast<uint64_t>(w3) << 32) | w2) >> 11, tau);
                     if (chosen < 0) {
                         fin = 1;                           // absorbing: nothing can fire
                     } else if (draws >= budget32) {
                         sh.status = PF_ST_BUDGET;
                         fin = 1;
                     } else {
-                        const double d = __dmul_rn(tau, fs.unit);
-                        t_next = t + static_cast<unsigned long long>(__double2ll_rn(fmin(d, 1.4411518807585587e17)));
+                        const double d = fmin(__dmul_rn(tau, fs.unit), 4503599627370496.0);
+                        const unsigned long long t = static_cast<unsigned long long>(__double2ll_rn(d)) + t_lo;
+                        n_hi = t_hi + static_cast<uint32_t>(t >> 30);
+                        n_lo = static_cast<uint32_t>(t) & 0x3FFFFFFFu;
                     }
                 }
                 if (fin) {
                     fired += draws;
                 } else {
                     ++draws;
-                    const uint32_t th = static_cast<uint32_t>(t_next >> 32);
-                    if (th >= quick_lo) {
-                        if (th > quick_hi) {
+                    if (n_hi >= quick_lo) {
+                        if (n_hi > quick_hi) {
                             fin = 1;
                         } else {
+                            const unsigned long long t = (static_cast<unsigned long long>(n_hi) << 30) | n_lo;
                             const unsigned long long b = fs.b0 + static_cast<unsigned long long>(fs.c) * draws +
                                                          static_cast<unsigned long long>(__float2ll_ru(err)) + 2ull;
-                            if (t_next > fs.D + b) fin = 1;
-                            else if (t_next + b >= fs.D) fin = 2;
+                            if (t > fs.D + b) fin = 1;
+                            else if (t + b >= fs.D) fin = 2;
                         }
                     }
                     if (fin == 0) {
-                        t = t_next;
+                        t_hi = n_hi;
+                        t_lo = n_lo;
                         const uint4 ch = fs.change[chosen];
                         auto apply = [&](uint32_t w) {
-                            int *p = reinterpret_cast<int *>(col + (w >> 16));
-                            *p += static_cast<int>(static_cast<int16_t>(w & 0xFFFFu));
+                            const uint32_t p = col + (w >> 16);
+                            col_store(p, col_load(p) + static_cast<uint32_t>(static_cast<int>(static_cast<int16_t>(w & 0xFFFFu))));
                         };
                         if (ch.x) apply(ch.x);
                         if (ch.y) {
@@ -535,11 +691,8 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
                 }
             }
             if (fin) {
-                if (fin == 1) {
-                    for (int u = 0; u < U; ++u) xs[u * Np + j] = *reinterpret_cast<int *>(col + u * 4 * B);
-                } else {
-                    redo[atomicAdd(&fs.n_exact, 1)] = j;
-                }
+                if (fin == 1) store_state();
+                else redo[atomicAdd(&fs.n_exact, 1)] = j;
                 active = false;
                 if (first) start(atomicAdd(&sh.pool_next, 1));
             }
@@ -552,6 +705,7 @@ __device__ __forceinline__ void ssa_fast(SharedHead &sh, FastShared &fs, int *co
         src = dst;
         first = false;
     }
+    return fired;
 }
 
 }  // namespace dev

@@ -45,11 +45,14 @@ struct ZigLayer {
 struct ZigTab {
     double x[kZigLayers + 1];
     ZigLayer layer[kZigLayers];
-    // for the path without FP64 (ssa_fast.cuh): x_i 2^-24 as a sum of two
-    // floats, and the largest t such that every draw whose first word's upper
-    // 16 bits lie in 16 .. 15 + t passes the layer's test
-    float fast_hi[kZigLayers], fast_lo[kZigLayers];
-    uint16_t fast_t[kZigLayers];
+    // for the path without FP64 (ssa_fast.cuh): x_i 2^-24 as a float plus the
+    // float whose upper 16 bits are fast_lo's; its lower 16 bits hold the largest
+    // t such that every draw whose first word's upper 16 bits lie in 16 .. 15 + t
+    // passes the layer's test
+    float fast_hi[kZigLayers];
+    uint32_t fast_lo[kZigLayers];
+    float wedge[kZigLayers];      // 1 / (exp(x_i - x_{i+1}) - 1)
+    uint64_t exp_t[kExpTable];    // exp(-i ln2 / 512) 2^63 (exp_neg_fixed)
 };
 
 // The shared-memory part: the layer edges the fast path reads.

@@ -92,3 +92,26 @@ def test_matches_the_oracle(name, N, cluster):
         assert (g["events"][ok] == o["events"][ok]).all()
         assert (g["digest"][ok] == o["digest"][ok]).all()
         np.testing.assert_allclose(g["loglik"][ok], o["loglik"][ok], rtol=1e-9, atol=0)
+
+
+@pytest.mark.parametrize("sigma", [1e-4, 0.05, 3.0, 1e7])
+@pytest.mark.parametrize("N", [1, 31, 32, 257, 700])
+def test_weights_match_the_oracle(sigma, N):
+    """The integer exponential of the weights: sharp densities (most weights
+    0 and far below 2^-62), flat ones (all near 1), the particles that attain
+    the maximum, several observed dimensions with coefficients and offsets."""
+    from paper_1606_08281_gb300 import pf
+    net = _net([({}, {0: 1}), ({0: 1}, {}), ({0: 1}, {1: 1})], 2)
+    thetas = np.array([[30.0, 0.5, 0.7], [4.0, 0.1, 0.1]])
+    times = np.array([0.0, 0.5, 1.0, 2.0])
+    C = np.array([[1.0, 0.0], [-0.25, 2.5]])
+    y = np.array([[[3.0, 1.0], [14.0, 20.0], [20.0, 40.0], [25.0, 60.0]]])
+    args = (net, thetas, np.array([3, 1], np.int32), times, y, C, np.array([sigma, 4 * sigma]), N, 17)
+    g = pf.pf_loglik(*args, diagnostics=True)
+    o = pf_oracle.pf_loglik(*args)
+    assert (g["status"] == o["status"]).all()
+    ok = o["status"] == 0
+    assert (g["digest"][ok] == o["digest"][ok]).all()
+    np.testing.assert_allclose(g["loglik"][ok], o["loglik"][ok], rtol=1e-12, atol=1e-12)
+    y[0, 1, 0] = np.nan
+    assert (pf.pf_loglik(*args)["status"] == pf.PF_ST_NONFINITE).all()
