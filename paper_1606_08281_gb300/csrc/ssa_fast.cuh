@@ -57,6 +57,8 @@ namespace dev {
 
 // Largest block of the filter kernels.
 constexpr int kMaxThreads = 256;
+// A warp parks at most kParkLanes - 1 particles a round.
+static_assert(kMaxThreads / 32 * (kParkLanes - 1) <= kMaxRemnants, "the parked particles' lists are too short");
 constexpr int kCheckTrips = 32;    // trips between two looks at the counts' caps
 
 // One reaction: A_r and the byte offsets of its reactants' rows in a column.
