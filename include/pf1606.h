@@ -112,8 +112,10 @@ typedef struct {
  *                 resampling / simulation history, used to compare paths.
  *   final_states  optional [M][T][N][U] particle states after the last
  *                 interval (int32).
- *   schedule      launch order of the filters: PF_SCHED_AUTO (currently row
- *                 order), PF_SCHED_NATURAL (row order), PF_SCHED_HEAVY_FIRST (a
+ *   schedule      launch order of the filters: PF_SCHED_AUTO (row order, or for
+ *                 launches of many long filters heaviest row first by the
+ *                 mean-field event counts), PF_SCHED_NATURAL (row order),
+ *                 PF_SCHED_HEAVY_FIRST (a
  *                 pilot path per theta row estimates its cost; rows run
  *                 heaviest first).  Results never depend on the order.
  *   row_order     optional [M] permutation of 0..M-1 (same memory space as

@@ -39,7 +39,7 @@ namespace dev {
 
 
 constexpr int kMaxWarps = 32;
-constexpr int kMaxRemnants = 128;  // >= block size
+constexpr int kMaxRemnants = 128;  // parked particles of a block
 constexpr int kParkLanes = 16;      // a warp below this many busy lanes parks its particles
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr uint32_t kResampleLane = 0xFFFFFFFFu;

@@ -139,25 +139,77 @@ __global__ void __launch_bounds__(128) pilot_kernel(const FilterArgs args, uint3
     cost[m] = events;
 }
 
-// Counting sort of theta rows by pilot cost, heaviest first (4 buckets per
+// Expected events of every theta row by the mean-field equations from x0 (FP32,
+// kMeanSteps steps to t_K; losses are taken implicitly, so that a stiff row
+// stays bounded): a cost estimate for scheduling only.  One thread per row,
+// about 20 us for four reactions.
+constexpr int kMeanSteps = 64;
+__global__ void __launch_bounds__(128) mean_field_kernel(const FilterArgs args, uint32_t *cost) {
+    __shared__ NetTables net;
+    {
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(&args.net);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&net);
+        for (int i = threadIdx.x; i < static_cast<int>(sizeof(NetTables) / 4); i += blockDim.x) dst[i] = src[i];
+    }
+    __syncthreads();
+    const int64_t m = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (m >= args.M) return;
+    const int R = net.R, U = net.U;
+    float rate[PF_MAX_REACTIONS], x[PF_MAX_SPECIES], gain[PF_MAX_SPECIES], loss[PF_MAX_SPECIES];
+    for (int r = 0; r < R; ++r) rate[r] = static_cast<float>(reaction_rate(net, args.thetas + m * net.d, r));
+    for (int u = 0; u < U; ++u) x[u] = 0.5f * (static_cast<float>(net.x0[u]) + static_cast<float>(net.x0_hi[u]));
+    const float dt = static_cast<float>(args.obs_times[args.K - 1]) / kMeanSteps;
+    float events = 0.0f;
+    for (int s = 0; s < kMeanSteps; ++s) {
+        for (int u = 0; u < U; ++u) gain[u] = loss[u] = 0.0f;
+        for (int r = 0; r < R; ++r) {
+            const int sa = net.sp_a[r], sb = net.sp_b[r];
+            float a = rate[r];
+            if (sa >= 0) a *= net.ord_a[r] == 2 ? 0.5f * x[sa] * x[sa] : x[sa];
+            if (sb >= 0) a *= x[sb];
+            events += a * dt;
+            for (int i = 0; i < net.n_change[r]; ++i) {
+                const int u = net.ch_sp[r][i];
+                const float c = a * static_cast<float>(net.ch_delta[r][i]);
+                if (c > 0.0f) gain[u] += c;
+                else loss[u] -= c;
+            }
+        }
+        for (int u = 0; u < U; ++u) x[u] = (x[u] + dt * gain[u]) / (1.0f + dt * loss[u] / fmaxf(x[u], 1e-3f));
+    }
+    // invalid rows and overflows order anywhere
+    cost[m] = events >= 0.0f && events < 4e9f ? static_cast<uint32_t>(events) : 0xFFFFFFFFu;
+}
+
+// Counting sort of theta rows by estimated cost, heaviest first (4 buckets per
 // octave).  One block.
 __global__ void __launch_bounds__(1024) order_kernel(const uint32_t *cost, int64_t M,
                                                       uint32_t *order) {
-    __shared__ int hist[64];
+    constexpr int kOrder = 128;
+    __shared__ int hist[kOrder];
     auto bucket = [](uint32_t c) {
         const int lg = c == 0 ? 0 : static_cast<int>(4.0f * __log2f(static_cast<float>(c)));
-        return 63 - min(63, max(0, lg));
+        return kOrder - 1 - min(kOrder - 1, max(0, lg));
     };
-    if (threadIdx.x < 64) hist[threadIdx.x] = 0;
+    if (threadIdx.x < kOrder) hist[threadIdx.x] = 0;
     __syncthreads();
     for (int64_t m = threadIdx.x; m < M; m += blockDim.x) atomicAdd(&hist[bucket(cost[m])], 1);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int b = 0; b < 64; ++b) {
-            const int c = hist[b];
-            hist[b] = run;
-            run += c;
+    if (threadIdx.x < 32) {                   // exclusive sums, four buckets a lane
+        int c[4], own = 0;
+        for (int i = 0; i < 4; ++i) {
+            c[i] = hist[4 * threadIdx.x + i];
+            own += c[i];
+        }
+        int run = own;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, run, o);
+            if (static_cast<int>(threadIdx.x) >= o) run += v;
+        }
+        run -= own;
+        for (int i = 0; i < 4; ++i) {
+            hist[4 * threadIdx.x + i] = run;
+            run += c[i];
         }
     }
     __syncthreads();
@@ -295,7 +347,8 @@ int launch_schedule(const FilterArgs &a, uint32_t *cost, uint32_t *order, uint32
     if (a.M == 0) return cudaSuccess;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const unsigned g = static_cast<unsigned>((a.M + 127) / 128);
-    switch (reaction_tier(a.net.R)) {
+    if (cap == 0) mean_field_kernel<<<g, 128, 0, s>>>(a, cost);
+    else switch (reaction_tier(a.net.R)) {
         case 4: pilot_kernel<4><<<g, 128, 0, s>>>(a, cost, cap); break;
         case 8: pilot_kernel<8><<<g, 128, 0, s>>>(a, cost, cap); break;
         case 16: pilot_kernel<16><<<g, 128, 0, s>>>(a, cost, cap); break;

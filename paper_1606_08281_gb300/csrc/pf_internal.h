@@ -119,7 +119,7 @@ double increment_slack(const NetTables &t);
 
 // Heaviest-first launch order of the theta rows: a pilot kernel simulates
 // one unconditioned path per row over [0, t_K] (its own random stream, at most
-// `cap` events) and a one-block counting sort orders rows by that event count.
+// `cap` events), or (cap = 0) integrates the mean-field equations, and a one-block counting sort orders rows by that event count.
 // cost [M] and order [M] are caller-provided device buffers.  The order only
 // affects scheduling, never results.
 int launch_schedule(const FilterArgs &a, uint32_t *cost, uint32_t *order, uint32_t cap,

@@ -115,3 +115,26 @@ def test_weights_match_the_oracle(sigma, N):
     np.testing.assert_allclose(g["loglik"][ok], o["loglik"][ok], rtol=1e-12, atol=1e-12)
     y[0, 1, 0] = np.nan
     assert (pf.pf_loglik(*args)["status"] == pf.PF_ST_NONFINITE).all()
+
+
+@pytest.mark.parametrize("name,N", [("gene_expression", 512), ("cascade", 64)])
+def test_launch_order_by_mean_field_does_not_change_results(name, N):
+    """PF_SCHED_AUTO's order (more filters than two per SM) against row order,
+    with rows that are invalid, zero and beyond any estimate among them."""
+    from paper_1606_08281_gb300 import pf
+    from paper_1606_08281_gb300 import workloads as W
+    w = W.get(name).subset(T=4, K=2)
+    th = w.thetas(90).copy()
+    th[3, 0] = -1.0
+    th[5] = 0.0
+    th[7, 0] = np.nan
+    th[9, 0] = 1e300
+    args = (w.net, th, w.x0, w.obs_times, w.observations(), w.C, w.sigma, N, 5)
+    a = pf.pf_loglik(*args, event_budget=4096, diagnostics=True)
+    b = pf.pf_loglik(*args, event_budget=4096, diagnostics=True, schedule=pf.PF_SCHED_NATURAL)
+    assert (a["status"] == b["status"]).all()
+    assert a["status"][3] == a["status"][7] == pf.PF_ST_INVALID_THETA
+    ok = a["status"] == 0
+    assert ok.sum() > 60
+    for k in ("loglik", "ll_traj", "events", "digest"):
+        assert (a[k][ok] == b[k][ok]).all()
