@@ -6,7 +6,7 @@ One *step* is one pf_loglik call over the whole gene-expression workload
 2 species / 4 reactions), inputs resident in HBM.  Reported:
   value        theta-likelihoods/s (whole job, all ranks),
   ssa_events_per_s, e2e (through the C ABI with host buffers, copies timed),
-  roofline     FP64 pipe of the filter kernel (the hot kernel),
+  roofline     instruction issue of the filter kernel (the hot kernel),
   cpu_baseline the oracle on the host cores, on a bounded sample.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -40,8 +40,16 @@ WORKLOAD = "gene_expression"
 # many-filter workloads fill the GPU with one block per filter.
 CLUSTER_BLOCKS = {"birth_death": 4, "lac_gfp": 4}
 L2_FLUSH_BYTES = 256 << 20          # > 129 MB L2
-# FP64 roofline of the filter kernel.  Nominal GB300 FP64 rate 1.25 TFLOP/s
-# at the 2070 MHz maximum SM clock over 152 SMs = 4 flops per SM per clock.
+# The filter kernel's bound is instruction issue: 4 warp instructions per SM and
+# clock.  Warp instructions per SSA event (all of the kernel's, divided by the
+# events of its launch), counted by ncu (smsp__inst_executed) on the same
+# networks: gene expression 244 rows x 12 times, 4.288e9 for 311 337 047 events;
+# cascade 76 rows x 8 times, 1.3058e10 for 582 126 036.
+WARP_INSTR_PER_EVENT = {"gene_expression": 4.288e9 / 311337047, "cascade": 1.3058e10 / 582126036}
+# FP64 work of the method as it is defined.  Nominal GB300 FP64 rate 1.25 TFLOP/s
+# at the 2070 MHz maximum SM clock over 152 SMs = 4 flops per SM per clock.  The
+# kernels take the SSA's decisions in integer and FP32 arithmetic, so this is a
+# measure of the work done per second, not of a pipe.
 FP64_FLOPS_PER_SM_CLK = 4.0
 N_SMS = 152
 SM_MAX_MHZ = 2070.0
@@ -540,8 +548,13 @@ def main() -> None:
     if rank == 0:
         fpe = flops_per_event(w.R)
         achieved = fpe * ev_step / (local_ms * 1e-3) / 1e12
-        ops_rate = ops_per_event(w.R) * ev_step / (local_ms * 1e-3) / 1e12
-        ops_peak = FP64_PEAK_TFLOPS / 2.0
+        issue_peak = 4.0 * N_SMS * SM_MAX_MHZ * 1e6 / 1e12
+        ipe = WARP_INSTR_PER_EVENT.get(w.name)
+        issued = None if ipe is None else ipe * ev_step / (local_ms * 1e-3) / 1e12
+        # the mean-field estimate and the row order precede the filter kernel
+        ordered = launch["schedule"] == pf.PF_SCHED_HEAVY_FIRST or (
+            launch["schedule"] == pf.PF_SCHED_AUTO and a.cluster <= 1 and M > 1 and M * w.T > 2 * N_SMS and
+            (w.N >= 512 or w.R > 4))
         value = world * M / (ms * 1e-3)
         h2d = th_np.nbytes + y_np.nbytes + w.obs_times.nbytes
         d2h = M * 8 + M
@@ -555,18 +568,19 @@ def main() -> None:
             "clocks": clk,
             "e2e": {"value": world * M / e2e_s, "unit": "theta-likelihoods/s",
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-            "gpu_launches": 2 * a.steps,
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                         "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
+            "gpu_launches": (4 if ordered else 2) * a.steps,
+            "roofline": {"bound": "alu", "achieved": issued, "peak": issue_peak,
+                         "unit": "T warp instructions/s", "frac": None if issued is None else issued / issue_peak,
                          "traffic": FILTER_TRAFFIC_BYTES if w.name == WORKLOAD and w.M == 4096 else None,
-                         "kernel": (f"filter_kernel_cluster (FP64 pipe; {a.cluster}-block clusters)"
-                                    if a.cluster > 1 else "filter_kernel (FP64 pipe)"),
-                         "flops_per_event": fpe,
-                         "fp64_ops_per_event": ops_per_event(w.R),
-                         "fp64_pipe_ops_frac": ops_rate / ops_peak,
-                         "peak_source": "nominal GB300 FP64 1.25 TFLOP/s = 4 flops/SM/clk x "
-                                        "152 SMs x 2070 MHz",
+                         "kernel": (f"filter_kernel_cluster (instruction issue; {a.cluster}-block clusters)"
+                                    if a.cluster > 1 else "filter_kernel (instruction issue)"),
+                         "warp_instr_per_event": WARP_INSTR_PER_EVENT.get(w.name),
+                         "peak_source": "4 warp instructions/SM/clk x 152 SMs x 2070 MHz",
                          "kernel_ms": local_ms},
+            "fp64_definition": {"flops_per_event": fpe, "fp64_ops_per_event": ops_per_event(w.R),
+                                "tflops": achieved,
+                                "note": "FP64 flops of the events as the method defines them, per second; "
+                                        "the kernel executes few of them"},
             "fp64_probe": probe,
             "phase_share": phases,
             "cpu_baseline": cpu,
@@ -673,18 +687,22 @@ def run_fsp(a, pf) -> None:
         times.append(e0.elapsed_time(e1))
     clk = clocks.stop()
     ms = float(np.mean(times))
-    ops = fsp_ops(w, th_np)
-    ops_rate = ops / (ms * 1e-3)
+    # fsp_ops counts the whole box; the kernels run on the reachable states with
+    # the inflows they have (telegraph: 549 operations per product instead of
+    # 1464) or on a window whose width depends on the row (not counted)
+    ops = fsp_ops(w, th_np) * 549 / 1464 if w.name == "telegraph" else None
+    ops_rate = ops / (ms * 1e-3) if ops else None
     peak_ops = FP64_PEAK_TFLOPS * 1e12 / 2.0          # one FP64 operation per lane per slot
     line = {"metric": "exact FSP theta-likelihoods/s", "mode": "fsp", "value": w.M / (ms * 1e-3),
             "unit": "theta-likelihoods/s", "n_gpus": 1, "steps": a.steps, "warmup": max(3, a.warmup),
             "ms_per_step": ms, "higher_is_better": True, "dtype": "f64", "data": "synthetic",
             "config": fsp_config(w),
             "clocks": clk,
-            "roofline": {"bound": "alu", "achieved": ops_rate / 1e12, "peak": peak_ops / 1e12,
-                         "unit": "T FP64 ops/s", "frac": ops_rate / peak_ops, "traffic": None,
-                         "kernel": "fsp_kernel (FP64 pipe; the probability vectors stay in "
-                                   "shared memory)",
+            "roofline": {"bound": "alu", "achieved": ops_rate / 1e12 if ops_rate else None,
+                         "peak": peak_ops / 1e12, "unit": "T FP64 ops/s",
+                         "frac": ops_rate / peak_ops if ops_rate else None, "traffic": None,
+                         "kernel": "fsp_compact_kernel / fsp_window_kernel (FP64 pipe; the probability "
+                                   "vectors stay in shared memory)",
                          "fp64_ops_per_step": ops},
             "cpu_baseline": (None if a.no_cpu_baseline
                              else exact_baseline("fsp", w.name, w.M, a.cpu_seconds))}

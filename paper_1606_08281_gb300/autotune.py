@@ -2,7 +2,8 @@
 
 For a problem shape (network tier, species, particles, observation times) it
 times pf_loglik on a sample of theta rows for each candidate block size (lanes
-per filter: 64, 96, 128) and launch order, and keeps the fastest.  Results are
+per filter: the library's choice, 64, 96, 128) and launch order, and keeps the
+fastest.  Results are
 cached in a JSON file keyed by the shape, so a serving process tunes once.
 Results never depend on these parameters, only the time does: the filters'
 histories are exact integer work, and the weights' sum is taken in chunks of
@@ -21,7 +22,7 @@ from . import pf
 
 DEFAULT_CACHE = Path(os.environ.get("PF1606_AUTOTUNE_CACHE",
                                     Path.home() / ".cache" / "pf1606" / "autotune.json"))
-BLOCKS = (64, 96, 128)
+BLOCKS = (0, 64, 96, 128)     # 0: the library's choice (256 from 512 particles on)
 
 
 def shape_key(net: dict, N: int, K: int, T: int) -> str:
@@ -56,7 +57,7 @@ def tune(net: dict, thetas, x0, obs_times, y, C, sigma, N: int, seed: int = 1, r
     y_d = torch.from_numpy(np.ascontiguousarray(y, dtype=np.float64)).to(dev)
     timings = {}
     for B in BLOCKS:
-        for sched in (pf.PF_SCHED_NATURAL, pf.PF_SCHED_HEAVY_FIRST):
+        for sched in (pf.PF_SCHED_AUTO, pf.PF_SCHED_NATURAL, pf.PF_SCHED_HEAVY_FIRST):
             def call():
                 pf.pf_loglik(net, th_d, x0, obs_times, y_d, C, sigma, N, seed, block_threads=B,
                              schedule=sched)
