@@ -33,6 +33,8 @@
  *     counter = (draw j, particle i, (trajectory << 20) | interval k, theta
  *     id); hence K < 2^20 and T < 2^12.
  *   - No function keeps a caller pointer after it returns.
+ *   - Device scratch is allocated in stream order from a memory pool of the
+ *     library that keeps at most 64 MiB per device between calls.
  */
 #ifndef PF1606_H
 #define PF1606_H

@@ -46,6 +46,38 @@ int cuda_fail(int err, const char *what) {
 
 void clear_error() { g_last_error.clear(); }
 
+// Scratch comes from a pool of the library's own that keeps up to 64 MiB per
+// device across synchronisations.  The default pool gives everything back at
+// each one, and mapping it again cost every call 200 us (one theta from host
+// memory 619 -> 426 us, the telegraph batch 2.94 -> 2.74 ms).
+int alloc_scratch(void **p, size_t bytes, cudaStream_t stream) {
+    constexpr int kDevices = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[kDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if (dev >= 0 && dev < kDevices) {
+        std::lock_guard<std::mutex> lock(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made = nullptr;
+            uint64_t keep = 64ull << 20;
+            if (cudaMemPoolCreate(&made, &props) == cudaSuccess) {
+                if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) pools[dev] = made;
+                else cudaMemPoolDestroy(made);
+            }
+            if (!pools[dev]) cudaGetLastError();      // no such pool: the default one serves
+        }
+        pool = pools[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, stream) : cudaMallocAsync(p, bytes, stream);
+}
+
 // Build the kernels' network tables from the caller's description.
 int build_tables(const pf_network *net, int32_t d, const int32_t *x0, int32_t P, const double *C,
                  const double *sigma, const pf_model *model, pf::NetTables &t) {
@@ -197,7 +229,7 @@ struct DevBuf {
     ~DevBuf() { if (p) cudaFreeAsync(p, s); }
     cudaError_t alloc(size_t bytes, cudaStream_t st) {
         s = st;
-        return bytes ? cudaMallocAsync(&p, bytes, st) : cudaSuccess;
+        return bytes ? static_cast<cudaError_t>(pf::alloc_scratch(&p, bytes, st)) : cudaSuccess;
     }
 };
 

@@ -754,7 +754,7 @@ struct Buf {
     ~Buf() { if (p) cudaFreeAsync(p, s); }
     cudaError_t alloc(size_t bytes, cudaStream_t st) {
         s = st;
-        return bytes ? cudaMallocAsync(&p, bytes, st) : cudaSuccess;
+        return bytes ? static_cast<cudaError_t>(alloc_scratch(&p, bytes, st)) : cudaSuccess;
     }
 };
 

@@ -125,6 +125,10 @@ double increment_slack(const NetTables &t);
 int launch_schedule(const FilterArgs &a, uint32_t *cost, uint32_t *order, uint32_t cap,
                     void *stream);
 
+// Stream-ordered scratch of a call (free with cudaFreeAsync); returns a
+// cudaError_t value.
+int alloc_scratch(void **p, size_t bytes, struct CUstream_st *stream);
+
 // Host-side validation helpers (pf_api.cu).  fail() records a message for
 // pf_last_error() and returns `code`.
 int fail(int code, const char *fmt, ...);

@@ -633,7 +633,7 @@ struct OBuf {
     ~OBuf() { if (p) cudaFreeAsync(p, s); }
     cudaError_t alloc(size_t bytes, cudaStream_t st) {
         s = st;
-        return bytes ? cudaMallocAsync(&p, bytes, st) : cudaSuccess;
+        return bytes ? static_cast<cudaError_t>(alloc_scratch(&p, bytes, st)) : cudaSuccess;
     }
 };
 
