@@ -406,7 +406,8 @@ typedef struct pf_ctx pf_ctx;
  *                     each slot owns its tables, stream and captured graph.
  *   max_particles     largest N a request may use (0 = 4096).
  * Allocates all slot memory up front.  A filter's population N (12 + 4U) + 16
- * bytes runs in a shared-memory arena sized for 4 blocks per SM if it fits,
+ * bytes runs in a shared-memory arena sized for 4 blocks per SM (3 for networks
+ * of more than 4 reactions or species) if it fits,
  * else in one sized for 2 blocks per SM, else in a global-memory slab (2
  * blocks per SM, as pf_loglik); the arenas are what the occupancy calculator
  * gives for the tier's kernel and block size.  Returns PF_OK, PF_EINVAL,

@@ -38,7 +38,7 @@ namespace {
 using namespace dev;
 
 constexpr int kTiers = 4;             // (R<=4,U<=4 in registers), R<=8, R<=16, R<=32
-// x {population in a shared-memory arena sized for 4 blocks per SM, in a global
+// x {population in a shared-memory arena sized for 4 or 3 blocks per SM, in a global
 //    slab, split over a thread-block cluster, in an arena sized for 2 blocks per SM}
 constexpr int kKinds = 4;
 constexpr int kGroups = kKinds * kTiers;
@@ -312,11 +312,11 @@ int tier_of(const NetTables &t) {
     return 3;
 }
 
-// Blocks per SM of the two on-chip kinds: the small arena keeps the filter
-// kernels' own occupancy (4 blocks of 128 threads: e.g. 512 particles of 10
-// species, 1300 of 2), the large one takes populations up to about 80 KB at 2
-// blocks per SM (e.g. 4096 particles of 2 species, 1500 of 10), as a plain
-// pf_loglik launch sized for them would.  Larger populations go to the slabs.
+// Blocks per SM of the two on-chip kinds, beside the head, tables and columns
+// of the SSA: the small arena leaves 4 blocks of 128 threads for small networks
+// (1000 particles of 2 species) and 3 for the others (650 of 10), the large one 2
+// (3900 of 2 species, 1380 of 10).  Larger populations go to the slabs, where
+// the SSA still runs in the columns.
 constexpr int kSmallArenaBlocks = 4, kLargeArenaBlocks = 2;
 
 // Shared memory ahead of a tier's population arena: the block's head and the

@@ -9,13 +9,12 @@
 // Within one interval the particles form a pool: each lane simulates one
 // particle and, when that particle reaches t_k, takes the next unclaimed one
 // (a shared-memory counter), so warps stay full although particles fire very
-// different numbers of reactions.  GB300's FP64 pipe spends the same 16
-// cycles on a warp instruction whatever its active-lane count, so idle lanes
-// would cost FP64 throughput directly.
-// The whole particle population lives in shared memory: states int32 [U][N]
-// (two buffers for the gather), the weights / integer-weight prefix sums
-// (8 bytes per particle, reused), and the ancestor indices.  Nothing of the
-// filter touches HBM between its first load and its final store.
+// different numbers of reactions.  The SSA's outcome is defined in FP64
+// (ssa_interval); ssa_fast.cuh reaches the same outcome without it and is what
+// almost every interval runs.  The whole particle population lives in shared
+// memory: states int32 [U][N], the weights / integer-weight prefix sums (8 bytes
+// per particle, reused), and the ancestor indices.  Nothing of the filter
+// touches HBM between its first load and its final store.
 //
 // Arithmetic that decides integer outcomes (propensities, their prefix sums,
 // event times, the Gaussian exponent) uses explicit round-to-nearest
@@ -815,9 +814,10 @@ __device__ __forceinline__ double log_weight(const SharedHead &sh, const int *xs
 // One filter -- one (theta row, observed trajectory) pair -- through all K
 // observation times (Supp. I, algorithm "Likelihood Approximation using particle
 // filter").  Called by every thread of the block.  Preconditions: sh.net and
-// sh.logt are loaded and a __syncthreads() has passed.  `arrays` holds the
-// particle population, N (16 + 8U) bytes (shared memory, or a per-block slab
-// of global memory for populations that do not fit on chip).
+// sh.zig_g (and, with `fast`, the ziggurat of ssa_fast.cuh) are loaded and a
+// __syncthreads() has passed.  `arrays` holds the particle population
+// (filter_smem_bytes; shared memory, or a per-block slab of global memory for
+// populations that do not fit on chip).
 struct FilterJob {
     const double *theta;      // [d] this filter's theta row
     const double *obs_times;  // [K]

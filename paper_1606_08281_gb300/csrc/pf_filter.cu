@@ -6,16 +6,7 @@
 // the blocks of a thread-block cluster instead (filter_kernel_cluster):
 //   resample by the previous weights -> simulate every particle to t_k with
 //   the direct-method SSA -> Gaussian weight -> log-sum-exp increment.
-// Within one interval the particles form a pool: each lane simulates one
-// particle and, when that particle reaches t_k, takes the next unclaimed one
-// (a shared-memory counter), so warps stay full although particles fire very
-// different numbers of reactions.  GB300's FP64 pipe spends the same 16
-// cycles on a warp instruction whatever its active-lane count, so idle lanes
-// would cost FP64 throughput directly.
-// The whole particle population lives in shared memory: states int32 [U][N]
-// (two buffers for the gather), the weights / integer-weight prefix sums
-// (8 bytes per particle, reused), and the ancestor indices.  Nothing of the
-// filter touches HBM between its first load and its final store.
+// (run_filter in pf_device.cuh).
 //
 // Arithmetic that decides integer outcomes (propensities, their prefix sums,
 // event times, the Gaussian exponent) uses explicit round-to-nearest

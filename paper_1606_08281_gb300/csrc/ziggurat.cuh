@@ -13,8 +13,8 @@
 // once in 50-digit arithmetic (the same equations reproduce the published
 // r = 7.69711747013104972 for 256 layers).  The host builds the table once
 // (build_zig_table) with the C library's exp/log and copies it to the device;
-// the kernels keep x_i in shared memory and read the rest (used by 0.34 % of
-// draws) from global memory.
+// ssa_fast.cuh keeps its form of the layers in shared memory, zig_exp reads the
+// table in global memory.
 #pragma once
 #include <cstdint>
 
